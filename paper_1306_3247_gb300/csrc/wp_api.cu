@@ -16,6 +16,7 @@
 
 #include "wp_fft_f64.h"
 #include "wp_ff.cuh"
+#include "wp_fx.h"
 #include "wp_internal.h"
 
 using namespace wp;
@@ -255,12 +256,14 @@ void host_twiddles(int64_t n, std::vector<double>& re, std::vector<double>& im) 
   }
 }
 
+// fx (or NULL): the factors without the scale, for the fixed-point passes.
 void host_kinetic(const wp_handle* h, int d, double tau, double scale, std::vector<double>& re,
-                  std::vector<double>& im) {
+                  std::vector<double>& im, std::vector<FxRec>* fx = nullptr) {
   const long double pi = 3.141592653589793238462643383279502884L;
   const int64_t n = h->n[d];
   re.resize(n);
   im.resize(n);
+  if (fx) fx->resize(n);
   const long double L = h->pb.L[d];
   for (int64_t j = 0; j < n; j++) {
     const int64_t js = j < n / 2 ? j : j - n;
@@ -269,6 +272,7 @@ void host_kinetic(const wp_handle* h, int d, double tau, double scale, std::vect
     th = fmodl(th, 2.0L * pi);
     re[j] = (double)(cosl(th) * (long double)scale);
     im[j] = (double)(sinl(th) * (long double)scale);
+    if (fx) (*fx)[j] = fx_rec_host(cosl(th), sinl(th));
   }
 }
 
@@ -335,6 +339,7 @@ wp_status alloc_tables(wp_handle* h) {
   size_t off_obs[3][3];
   size_t off_w256[3] = {0, 0, 0};
   size_t off_w2s[3] = {0, 0, 0};
+  size_t off_fx[3][4] = {};
   for (int d = 0; d < h->ndim; d++) {
     const size_t n = (size_t)h->n[d];
     for (int k = 0; k < 4; k++) off[d][k] = add(n * sizeof(cx<T>));
@@ -352,6 +357,8 @@ wp_status alloc_tables(wp_handle* h) {
     off_obs[d][2] = add(n * sizeof(T));
     off_w256[d] = (!std::is_same<T, double>::value && n == 256) ? add(256 * 16) : 0;
     off_w2s[d] = (std::is_same<T, float>::value && (n == 64 || n == 128)) ? add(256 * 16) : 0;
+    if (std::is_same<T, double>::value)
+      for (int k = 0; k < 4; k++) off_fx[d][k] = add(n * sizeof(FxRec));
   }
   WP_CUDA(h, dev_malloc(h, &h->tabmem, bytes));
   WP_CUDA(h, cudaMemsetAsync(h->tabmem, 0, bytes, h->stream));
@@ -380,6 +387,12 @@ wp_status alloc_tables(wp_handle* h) {
     tb[d].W256 = (!std::is_same<T, double>::value && h->n[d] == 256) ? (void*)(base + off_w256[d]) : nullptr;
     tb[d].W2s = (std::is_same<T, float>::value && (h->n[d] == 64 || h->n[d] == 128)) ? (void*)(base + off_w2s[d])
                                                                                      : nullptr;
+    if (std::is_same<T, double>::value) {
+      tb[d].Wfx = (FxRec*)(base + off_fx[d][0]);
+      tb[d].Kfx_full = (FxRec*)(base + off_fx[d][1]);
+      tb[d].Kfx_half = (FxRec*)(base + off_fx[d][2]);
+      tb[d].Pfx = (FxRec*)(base + off_fx[d][3]);
+    }
   }
   // static tables (high and low parts)
   for (int d = 0; d < h->ndim; d++) {
@@ -413,6 +426,7 @@ wp_status alloc_tables(wp_handle* h) {
       // then (FP32 only) low part
       const int logn = h->g.ln[d];
       std::vector<unsigned char> rec(n * 16, 0);
+      std::vector<FxRec> fx(tb[d].Wfx ? n : 0, FxRec{});
       const long double pi = 3.141592653589793238462643383279502884L;
       int ls = 0;
       while (ls < logn) {
@@ -429,11 +443,13 @@ wp_status alloc_tables(wp_handle* h) {
               unsigned char* dst = &rec[(size_t)(off + jm * ((1 << lr) - 1) + r - 1) * 16];
               memcpy(dst, &rh, sizeof(rh));
               if (sizeof(cx<T>) == 8) memcpy(dst + 8, &rl, sizeof(rl));
+              if (!fx.empty()) fx[(size_t)(off + jm * ((1 << lr) - 1) + r - 1)] = fx_rec_host(cosl(a), sinl(a));
             }
         }
         ls += lr;
       }
       WP_CUDA(h, cudaMemcpy(tb[d].Wst, rec.data(), rec.size(), cudaMemcpyHostToDevice));
+      if (!fx.empty()) WP_CUDA(h, cudaMemcpy(tb[d].Wfx, fx.data(), n * sizeof(FxRec), cudaMemcpyHostToDevice));
     }
     if (tb[d].W256) {
       // two-stage 256-point kernels: exp(-2 pi i t k1/256) at k1 * 16 + t (complex64: high +
@@ -481,20 +497,34 @@ wp_status alloc_tables(wp_handle* h) {
     }
     const double scale = d == 0 ? 1.0 / (double)h->N : 1.0;
     std::vector<TwE<T>> recs(n);
-    host_kinetic(h, d, h->pb.dt, scale, re, im);
+    std::vector<FxRec> fx;
+    std::vector<FxRec>* const pfx = std::is_same<T, double>::value ? &fx : nullptr;
+    host_kinetic(h, d, h->pb.dt, scale, re, im, pfx);
     split();
+    if (pfx) WP_CUDA(h, cudaMemcpy(tb[d].Kfx_full, fx.data(), n * sizeof(FxRec), cudaMemcpyHostToDevice));
     for (size_t k = 0; k < n; k++) recs[k] = make_rec<T>(re[k], im[k]);
     WP_CUDA(h, cudaMemcpy(tb[d].Kfull, hi.data(), nb, cudaMemcpyHostToDevice));
     WP_CUDA(h, cudaMemcpy(tb[d].Kfull_lo, lo.data(), nb, cudaMemcpyHostToDevice));
     WP_CUDA(h, cudaMemcpy(tb[d].Kfull_rec, recs.data(), n * sizeof(TwE<T>), cudaMemcpyHostToDevice));
-    host_kinetic(h, d, 0.5 * h->pb.dt, scale, re, im);
+    host_kinetic(h, d, 0.5 * h->pb.dt, scale, re, im, pfx);
     split();
+    if (pfx) WP_CUDA(h, cudaMemcpy(tb[d].Kfx_half, fx.data(), n * sizeof(FxRec), cudaMemcpyHostToDevice));
     for (size_t k = 0; k < n; k++) recs[k] = make_rec<T>(re[k], im[k]);
     WP_CUDA(h, cudaMemcpy(tb[d].Khalf, hi.data(), nb, cudaMemcpyHostToDevice));
     WP_CUDA(h, cudaMemcpy(tb[d].Khalf_lo, lo.data(), nb, cudaMemcpyHostToDevice));
     WP_CUDA(h, cudaMemcpy(tb[d].Khalf_rec, recs.data(), n * sizeof(TwE<T>), cudaMemcpyHostToDevice));
   }
   return WP_OK;
+}
+
+// Whether every pass of a step runs in fixed point, so that the state may stay in it between
+// them: complex128, fixed-shape plans on every axis and no grid potential (its passes are
+// FP64).
+bool fx_state(const wp_handle* h) {
+  if (h->prec != WP_C128 || h->ndim < 2 || h->vgrid) return false;
+  for (int d = 0; d < h->ndim; d++)
+    if (!h->plan[d].fixed) return false;
+  return true;
 }
 
 // ------------------------------------------------------------------ launches
@@ -556,6 +586,11 @@ PassParams<T> pass_params(wp_handle* h, int axis, uint32_t flags, void* in, void
   p.grid_rec = (h->vgrid && h->phase_half >= 0) ? (const TwE<T>*)h->vgrid_rec[h->phase_half] : nullptr;
   p.W256 = tb[axis].W256;
   p.W2s = tb[axis].W2s;
+  p.Wfx = tb[axis].Wfx;
+  p.Pfx = tb[axis].Pfx;
+  p.Kfx = khalf ? tb[axis].Kfx_half : tb[axis].Kfx_full;
+  p.Kfx_half = tb[axis].Kfx_half;
+  p.fx_state = fx_state(h) ? 1 : 0;
   return p;
 }
 
@@ -855,9 +890,9 @@ template <class T>
 wp_status momentum_and_reduce(wp_handle* h) {
   wp_status st;
   const int nd = h->ndim;
-  if ((st = run_pass<T>(h, nd - 1, F_FFT, h->state, h->scratch)) != WP_OK) return st;
+  if ((st = run_pass<T>(h, nd - 1, F_FFT | (nd == 3 ? F_OUT_FX : 0u), h->state, h->scratch)) != WP_OK) return st;
   if (nd == 3)
-    if ((st = run_pass<T>(h, 1, F_FFT, h->scratch, h->scratch)) != WP_OK) return st;
+    if ((st = run_pass<T>(h, 1, F_FFT | F_IN_FX, h->scratch, h->scratch)) != WP_OK) return st;
   if ((st = run_pass<T>(h, 0, F_FFT | F_OBS_MOM | F_NO_STORE, h->scratch, h->scratch, h->part_mom)) != WP_OK)
     return st;
   ReduceParams r{};
@@ -928,43 +963,47 @@ wp_status chunk_seq(wp_handle* h, int64_t m, bool obs_end) {
   }
   void* S = h->state;
   const int Z = nd - 1;
-  auto middle = [&](int khalf) -> wp_status {
+  // between the passes of the chunk a complex128 state is in fixed point (fx_state); a pass
+  // that forms observable sums is FP64 and reads doubles
+  constexpr uint32_t FX = F_IN_FX | F_OUT_FX;
+  auto middle = [&](int khalf, bool to_fx) -> wp_status {
     wp_status s2;
+    const uint32_t last = F_IN_FX | (to_fx ? F_OUT_FX : 0u);
     if (nd == 3)
-      if ((s2 = run_pass<T>(h, 1, F_FFT, S, S)) != WP_OK) return s2;
-    if ((s2 = run_pass<T>(h, 0, F_KIN, S, S, nullptr, khalf)) != WP_OK) return s2;
+      if ((s2 = run_pass<T>(h, 1, F_FFT | FX, S, S)) != WP_OK) return s2;
+    if ((s2 = run_pass<T>(h, 0, F_KIN | (nd == 3 ? FX : last), S, S, nullptr, khalf)) != WP_OK) return s2;
     if (nd == 3)
-      if ((s2 = run_pass<T>(h, 1, F_IFFT, S, S)) != WP_OK) return s2;
+      if ((s2 = run_pass<T>(h, 1, F_IFFT | last, S, S)) != WP_OK) return s2;
     return WP_OK;
   };
-  const uint32_t obsf = obs_end ? (F_OBS_POS | (h->pb.autocorr ? F_AUTOCORR : 0u)) : 0u;
+  const uint32_t obsf = obs_end ? (F_OBS_POS | (h->pb.autocorr ? F_AUTOCORR : 0u)) : F_IN_FX;
   // the tables of step k + 1 are formed beside the strided passes of step k
   if (h->pb.order == WP_ORDER_VKV) {
     if ((st = run_prep<T>(h, 0, 0.0, 0.5 * dt, true)) != WP_OK) return st;
-    if ((st = run_pass<T>(h, Z, F_PHASE | F_FFT, S, S)) != WP_OK) return st;
+    if ((st = run_pass<T>(h, Z, F_PHASE | F_FFT | F_OUT_FX, S, S)) != WP_OK) return st;
     for (int64_t k = 1; k < m; k++) {
       if ((st = fork_tables<T>(h, 1, 0.0, dt, true)) != WP_OK) return st;
-      if ((st = middle(0)) != WP_OK) return st;
+      if ((st = middle(0, true)) != WP_OK) return st;
       if ((st = join_tables(h)) != WP_OK) return st;
-      if ((st = run_pass<T>(h, Z, F_IFFT | F_PHASE | F_FFT, S, S)) != WP_OK) return st;
+      if ((st = run_pass<T>(h, Z, F_IFFT | F_PHASE | F_FFT | FX, S, S)) != WP_OK) return st;
     }
     if ((st = fork_tables<T>(h, 1, 0.0, 0.5 * dt, true)) != WP_OK) return st;
-    if ((st = middle(0)) != WP_OK) return st;
+    if ((st = middle(0, !obs_end)) != WP_OK) return st;
     if ((st = join_tables(h)) != WP_OK) return st;
     if ((st = run_pass<T>(h, Z, F_IFFT | F_PHASE | obsf, S, S, h->part_pos)) != WP_OK) return st;
   } else {
-    if ((st = run_pass<T>(h, Z, F_FFT, S, S)) != WP_OK) return st;
+    if ((st = run_pass<T>(h, Z, F_FFT | F_OUT_FX, S, S)) != WP_OK) return st;
     if ((st = fork_tables<T>(h, 0, 0.5 * dt, dt, true)) != WP_OK) return st;
-    if ((st = middle(1)) != WP_OK) return st;
+    if ((st = middle(1, true)) != WP_OK) return st;
     for (int64_t k = 0; k < m; k++) {
       if ((st = join_tables(h)) != WP_OK) return st;
-      if ((st = run_pass<T>(h, Z, F_IFFT | F_PHASE | F_FFT, S, S)) != WP_OK) return st;
+      if ((st = run_pass<T>(h, Z, F_IFFT | F_PHASE | F_FFT | FX, S, S)) != WP_OK) return st;
       if (k < m - 1) {
         if ((st = fork_tables<T>(h, 1, 0.5 * dt, dt, true)) != WP_OK) return st;
       } else {
         if ((st = fork_tables<T>(h, 1, 0.0, 0.0, false)) != WP_OK) return st;
       }
-      if ((st = middle(k == m - 1 ? 1 : 0)) != WP_OK) return st;
+      if ((st = middle(k == m - 1 ? 1 : 0, k < m - 1 || !obs_end)) != WP_OK) return st;
     }
     if ((st = join_tables(h)) != WP_OK) return st;
     if ((st = run_pass<T>(h, Z, F_IFFT | obsf, S, S, h->part_pos)) != WP_OK) return st;
@@ -1413,6 +1452,7 @@ wp_status batch_compile(wp_batch* b) {
 template <class T>
 wp_status batch_issue(wp_batch* b, int64_t m) {
   cudaStream_t st = b->stream;
+  constexpr uint32_t FX = F_IN_FX | F_OUT_FX;  // between the passes of the chunk, as chunk_seq
   const int n2 = (int)b->idx2d.size();
   auto prep = [&](int add, double shift, double tau) -> wp_status {
     b->launches++;
@@ -1460,7 +1500,7 @@ wp_status batch_issue(wp_batch* b, int64_t m) {
       b->launches++;
       const wp_status r = launch_rc(
           nullptr,
-          launch_merged_strided<T>((const PassParams<T>*)b->d_pass_x, b->d_tiles_x, b->d_binst_x, ml, F_KIN, khalf,
+          launch_merged_strided<T>((const PassParams<T>*)b->d_pass_x, b->d_tiles_x, b->d_binst_x, ml, F_KIN | FX, khalf,
                                    (const PrepParams<T>*)b->d_prep, (const LinesParams<T>*)b->d_lines,
                                    b->smem_merged, st),
           "batched pass");
@@ -1470,7 +1510,7 @@ wp_status batch_issue(wp_batch* b, int64_t m) {
       b->launches++;
       const wp_status r = launch_rc(nullptr,
                                     launch_pass_batch<T>((const PassParams<T>*)b->d_pass_x, b->d_tiles_x, b->d_binst_x,
-                                                         c.logn, c.off, c.n, F_KIN, khalf, b->smem2d, st),
+                                                         c.logn, c.off, c.n, F_KIN | FX, khalf, b->smem2d, st),
                                     "batched pass");
       if (r != WP_OK) return r;
     }
@@ -1501,22 +1541,22 @@ wp_status batch_issue(wp_batch* b, int64_t m) {
     // each one launch for the Stockham classes plus one per class of its own (the order
     // of tables, potential and kinetic passes is unchanged)
     if (b->order2d == WP_ORDER_VKV) {
-      if ((s2 = prep(0, 0.0, 0.5)) != WP_OK || (s2 = zmerged(F_PHASE | F_FFT)) != WP_OK) return s2;
+      if ((s2 = prep(0, 0.0, 0.5)) != WP_OK || (s2 = zmerged(F_PHASE | F_FFT | F_OUT_FX)) != WP_OK) return s2;
       for (int64_t k = 1; k < m; k++)
-        if ((s2 = xmerged(0, true, 1, 0.0, 1.0)) != WP_OK || (s2 = zmerged(F_IFFT | F_PHASE | F_FFT)) != WP_OK)
+        if ((s2 = xmerged(0, true, 1, 0.0, 1.0)) != WP_OK || (s2 = zmerged(F_IFFT | F_PHASE | F_FFT | FX)) != WP_OK)
           return s2;
-      if ((s2 = xmerged(0, true, 1, 0.0, 0.5)) != WP_OK || (s2 = zmerged(F_IFFT | F_PHASE)) != WP_OK) return s2;
+      if ((s2 = xmerged(0, true, 1, 0.0, 0.5)) != WP_OK || (s2 = zmerged(F_IFFT | F_PHASE | F_IN_FX)) != WP_OK) return s2;
     } else {
-      if ((s2 = zmerged(F_FFT)) != WP_OK || (s2 = xmerged(1, true, 0, 0.5, 1.0)) != WP_OK) return s2;
+      if ((s2 = zmerged(F_FFT | F_OUT_FX)) != WP_OK || (s2 = xmerged(1, true, 0, 0.5, 1.0)) != WP_OK) return s2;
       for (int64_t k = 0; k < m; k++) {
-        if ((s2 = zmerged(F_IFFT | F_PHASE | F_FFT)) != WP_OK) return s2;
+        if ((s2 = zmerged(F_IFFT | F_PHASE | F_FFT | FX)) != WP_OK) return s2;
         if (k < m - 1)
           s2 = xmerged(0, true, 1, 0.5, 1.0);
         else
           s2 = xmerged(1, true, 1, 0.0, 0.0);
         if (s2 != WP_OK) return s2;
       }
-      if ((s2 = zmerged(F_IFFT)) != WP_OK) return s2;
+      if ((s2 = zmerged(F_IFFT | F_IN_FX)) != WP_OK) return s2;
     }
   }
   for (int k : b->idx_other) {

@@ -105,9 +105,9 @@ __device__ __forceinline__ void merged_class_body(int key, const PassParams<T>* 
 
 template <class T>
 constexpr int merged_min_blocks() {
-  // complex64: five blocks per SM (the single-class kernels took 32-48 registers); FP64
-  // the four of its fixed-shape batched kernels; float-float three
-  return std::is_same<T, float>::value ? 5 : (std::is_same<T, ff>::value ? 3 : 4);
+  // complex64: five blocks per SM (the single-class kernels took 32-48 registers);
+  // complex128 and float-float three
+  return std::is_same<T, float>::value ? 5 : 3;
 }
 
 // CONTIG: the potential pass (axis 1) or the kinetic pass (axis 0). Launch blocks

@@ -11,10 +11,13 @@
 namespace wp {
 namespace fixed_detail {
 
-// The kernel of a shape: the FP64 one has its own register bound.
+// The kernel of a shape: complex128 passes without sums or a grid in fixed point, the others
+// in FP64 with their own register bound.
 template <class T, int LOGN, bool CONTIG, bool OBS, bool GRID>
 constexpr auto kernel_of() {
-  if constexpr (std::is_same<T, double>::value)
+  if constexpr (std::is_same<T, double>::value && !OBS && !GRID)
+    return &fxp::k_pass_fx<LOGN, CONTIG>;
+  else if constexpr (std::is_same<T, double>::value)
     return &k_pass_fixed_f64<LOGN, CONTIG, OBS, GRID>;
   else
     return &k_pass_fixed<T, LOGN, CONTIG, OBS, GRID>;

@@ -19,6 +19,8 @@ enum PassFlags : uint32_t {
   F_OBS_MOM = 1u << 5,   // momentum-space partial sums (after the forward FFT)
   F_NO_STORE = 1u << 6,  // keep the tile (used by the momentum sums)
   F_AUTOCORR = 1u << 7,  // add <psi0|psi> to the position sums
+  F_IN_FX = 1u << 8,     // complex128, PassParams::fx_state: the pass reads fixed-point points
+  F_OUT_FX = 1u << 9,    // and writes them (wp_fx.h) instead of doubles
 };
 
 // Partial-sum slots per CTA.
@@ -88,6 +90,13 @@ __host__ __device__ inline TwE<float> make_rec<float>(double re, double im) {
   r.l = cx<float>{(float)(re - (double)hr), (float)(im - (double)hi)};
   return r;
 }
+
+// A unit factor c + i s of the fixed-point transforms (wp_fx.h): c, c + s and c - s times
+// 2^62, each as a high word and a signed low word. bad: the factor is not finite.
+struct alignas(16) FxRec {
+  int32_t ch, cl, ph, pl, mh, ml;
+  int32_t bad, reserved;
+};
 
 // Per-line record of a pass: the product of the other axes' factors (potential phase in
 // the contiguous pass, kinetic factor in the kinetic pass) and, for the potential, the
@@ -161,6 +170,12 @@ struct AxisTab {
   T* AT;                      // A(x,t) rounded to T: line sums of the potential energy
   void* W256;                 // complex64 and float-float, n = 256: records exp(-2 pi i t k1/256) at k1 * 16 + t
   void* W2s;                  // complex64, n = 64 or 128: two-stage twiddle records (wp_pass2s.cuh)
+  // complex128: the fixed-point factors (wp_fx.h). Stage twiddles (at the offsets of Wst),
+  // kinetic factors without the 1/N of axis 0, and the potential phase factors of the step.
+  FxRec* Wfx;
+  FxRec* Kfx_full;
+  FxRec* Kfx_half;
+  FxRec* Pfx;
 };
 
 template <class T>
@@ -210,6 +225,12 @@ struct PassParams {
   const double* grid_v;    // static grid potential (observables), or NULL
   const void* W256;        // two-stage 256-point kernels: twiddle records of the pass axis, or NULL
   const void* W2s;         // two-stage 64- and 128-point kernels: twiddle records, or NULL
+  // complex128: the pass axis's fixed-point factors (AxisTab)
+  const FxRec* Wfx;
+  const FxRec* Pfx;
+  const FxRec* Kfx;
+  const FxRec* Kfx_half;
+  int32_t fx_state;        // every pass of a step runs in fixed point: F_IN_FX, F_OUT_FX apply
 };
 
 // Per-line records of one pass (k_lines).

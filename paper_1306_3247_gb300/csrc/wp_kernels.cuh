@@ -17,6 +17,7 @@
 #include <type_traits>
 
 #include "wp_fft_f64.h"
+#include "wp_fx.h"
 #include "wp_ff.cuh"
 #include "wp_phase_ff.cuh"
 #include "wp_internal.h"
@@ -1171,6 +1172,12 @@ __device__ __forceinline__ void pass_body(const PassParams<T>& p, const SH& sh, 
   pass_compute<T, E, OBS, SH, GRID>(p, sh, s, tile);
 }
 
+// The complex128 passes in fixed point (wp_fx_pass.cuh).
+namespace fxp {
+template <int LOGN, bool CONTIG>
+__device__ __forceinline__ void pass(const PassParams<double>& p, cx<int64_t>* s, int64_t tile, cx<double> (&v)[8]);
+}  // namespace fxp
+
 // E elements per thread; the block has at most 32 E threads, so a tile holds at most
 // 32 E^2 elements (2048 for E = 8, 8192 for E = 16). OBS compiles the partial sums in.
 template <class T, int E, bool OBS>
@@ -1233,12 +1240,15 @@ __device__ __forceinline__ void pass_batch_body(const PassParams<T>* __restrict_
         p.K_lo[d] = p.Khalf_lo_axes[d];
       }
       p.Krec = p.Krec_half;
+      p.Kfx = p.Kfx_half;
       p.lines_kin = p.lines_kin_half;
     }
   }
   __syncthreads();
   cx<T>* s = reinterpret_cast<cx<T>*>(smem_raw);
-  if constexpr (LOGN > 0) {
+  if constexpr (LOGN > 0 && std::is_same<T, double>::value) {
+    fxp::pass<LOGN, CONTIG>(p, reinterpret_cast<cx<int64_t>*>(smem_raw), tile, v);
+  } else if constexpr (LOGN > 0) {
     using SH = FixShape<LOGN, CONTIG>;
     constexpr int ISTEP = 256 >> SH::logC;
 #pragma unroll
@@ -1267,10 +1277,10 @@ __global__ void __launch_bounds__(256) k_pass_batch(const PassParams<T>* __restr
   __shared__ __align__(16) unsigned char raw[sizeof(PassParams<T>)];
   pass_batch_body<T, CONTIG, LOGN>(params, tile_start, block_inst, block_off + blockIdx.x, flags, khalf, raw);
 }
-// FP64 with a compile-time shape (LOGN = 6..10): at most 64 registers, so that four
-// blocks share an SM (the FP64 pipe needs the warps to cover its latency).
+// complex128 with a compile-time shape (LOGN = 6..10): the fixed-point pass, three blocks
+// per SM as alone.
 template <bool CONTIG, int LOGN>
-__global__ void __launch_bounds__(256, 4) k_pass_batch_f64(const PassParams<double>* __restrict__ params,
+__global__ void __launch_bounds__(256, 3) k_pass_batch_f64(const PassParams<double>* __restrict__ params,
                                                           const int64_t* __restrict__ tile_start,
                                                           const int* __restrict__ block_inst, int64_t block_off,
                                                           uint32_t flags, int khalf) {
@@ -1308,6 +1318,13 @@ __global__ void __launch_bounds__(256, (OBS || GRID) ? 3 : 4) k_pass_fixed_f64(c
   extern __shared__ __align__(16) unsigned char smem_raw[];
   pass_body<double, 8, OBS, FixShape<LOGN, CONTIG>, GRID>(p, FixShape<LOGN, CONTIG>(),
                                                           reinterpret_cast<cx<double>*>(smem_raw));
+}
+
+// The fixed-point record of a factor formed in FP64.
+__device__ __forceinline__ FxRec fx_rec_of(double c, double s) {
+  FxRec r = fx_rec(__double2ll_rn(c * 0x1p62), __double2ll_rn(s * 0x1p62));
+  r.bad = !isfinite(c);
+  return r;
 }
 
 // ------------------------------------------------------------------ per-line records
@@ -1405,6 +1422,7 @@ __device__ void prep_body(const PrepParams<T>& p, int blk, int nblk) {
         tb.P[i] = mk(hc, hs);
         tb.P_lo[i] = mk((T)(cs - (double)hc), (T)(sn - (double)hs));
         tb.Prec[i] = make_rec<T>(cs, sn);
+        if constexpr (std::is_same<T, double>::value) tb.Pfx[i] = fx_rec_of(cs, sn);
       }
       for (int gg = 0; gg < pot.ngauss; gg++) {
         const double gf = gauss_axis_factor(pot.term[pot.gauss_term[gg]], d, x, t);
@@ -1904,3 +1922,5 @@ __global__ void k_gaussian(const GaussParams<T> p, int64_t ntotal) {
 }
 
 }  // namespace wp
+
+#include "wp_fx_pass.cuh"
