@@ -89,6 +89,8 @@ struct wp_handle {
   size_t res_smem = 0;
   bool res_fixed = false;          // 1-D line of compile-time length (k_res1d_fixed)
   void* res_S = nullptr;           // 1-D static phase tables, 2 x n records (dt, dt/2)
+  FxRec* res_Sfx = nullptr;        // complex128: the same in fixed point,
+  double* res_Vs = nullptr;        // and the static potential
   void* gauss_tab = nullptr;       // per-axis factors of the initial Gaussian
   double* vgrid = nullptr;         // static grid potential (FP64, N values), or NULL
   void* vgrid_rec[2] = {nullptr, nullptr};  // its phase records for dt, dt/2 (2-D, 3-D)
@@ -820,6 +822,12 @@ Res1dParams<T> res1d_params(wp_handle* h) {
   p.Wst = tb[0].Wst;
   p.Krec[0] = tb[0].Kfull_rec;
   p.Krec[1] = tb[0].Khalf_rec;
+  p.Wfx = tb[0].Wfx;
+  p.Kfx[0] = tb[0].Kfx_full;
+  p.Kfx[1] = tb[0].Kfx_half;
+  p.Sfx[0] = h->res_Sfx;
+  p.Sfx[1] = h->res_Sfx ? h->res_Sfx + h->n[0] : nullptr;
+  p.Vs = h->res_Vs;
   return p;
 }
 
@@ -836,6 +844,9 @@ wp_status res1d_static_tables(wp_handle* h, uint32_t stat) {
   sp.vgrid = h->vgrid;
   sp.S[0] = (TwE<T>*)h->res_S;
   sp.S[1] = (TwE<T>*)h->res_S + h->n[0];
+  sp.Sfx[0] = h->res_Sfx;
+  sp.Sfx[1] = h->res_Sfx ? h->res_Sfx + h->n[0] : nullptr;
+  sp.Vs = h->res_Vs;
   const int rc = launch_static_phase<T>(sp, h->stream);
   if (rc) return cuda_fail(h, (cudaError_t)rc, "static phase kernel");
   return WP_OK;
@@ -1740,6 +1751,11 @@ wp_status wp_create_pooled(const wp_problem* pb, void* stream, void* mem_pool, w
   if (h->ndim == 1) {
     if ((e = dev_malloc(h, &h->res_S, 2 * (size_t)h->n[0] * sizeof(TwE<double>))) != cudaSuccess)
       return bail(cuda_fail(h, e, "static phase allocation"));
+    if (h->prec == WP_C128) {
+      if ((e = dev_malloc(h, (void**)&h->res_Sfx, 2 * (size_t)h->n[0] * sizeof(FxRec))) != cudaSuccess ||
+          (e = dev_malloc(h, (void**)&h->res_Vs, (size_t)h->n[0] * sizeof(double))) != cudaSuccess)
+        return bail(cuda_fail(h, e, "static phase allocation"));
+    }
     if ((st = res1d_split_potential(h)) != WP_OK) return bail(st);
   }
   if ((st = ensure_obs(h, 64)) != WP_OK) return bail(st);
@@ -1754,7 +1770,7 @@ wp_status wp_destroy(wp_handle* h) {
   graphs_clear(h);
   void* ptrs[] = {h->state,    h->scratch,  h->psi0,     h->staging,     h->ctrl,          h->dpot,
                   h->tabmem,   h->part_pos, h->part_mom, h->obs_dev,     h->lines_phase,   h->lines_kin[0],
-                  h->lines_kin[1], h->res_S, h->gauss_tab, h->vgrid, h->vgrid_rec[0], h->vgrid_rec[1]};
+                  h->lines_kin[1], h->res_S, h->res_Sfx, h->res_Vs, h->gauss_tab, h->vgrid, h->vgrid_rec[0], h->vgrid_rec[1]};
   for (void* p : ptrs) dev_free(h, p);
   if (h->pool) cudaStreamSynchronize(h->stream);
   for (auto& ep : h->pending) {

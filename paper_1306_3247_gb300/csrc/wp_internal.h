@@ -295,6 +295,12 @@ struct Res1dParams {
   int32_t max_radix_log;     // largest butterfly of the run-time-length kernel (2 or 3)
   const void* Wst;           // per-stage twiddle records (fixed)
   const TwE<T>* Krec[2];     // kinetic factors dt, dt/2 as records (fixed)
+  // complex128 (fixed, wp_res1d_fx.cuh): fixed-point twiddles, kinetic factors without 1/n
+  // and static phases (dt, dt/2), and the static potential itself (observables)
+  const FxRec* Wfx;
+  const FxRec* Kfx[2];
+  const FxRec* Sfx[2];
+  const double* Vs;
 };
 
 // Static phase tables of a 1-D handle (k_static_phase), formed in FP64 and stored as records.
@@ -306,6 +312,8 @@ struct StaticPhaseParams {
   uint32_t static_mask;
   const double* vgrid; // static grid potential added to V_s, or NULL
   TwE<T>* S[2];        // exp(-i V_s dt / hbar), exp(-i V_s (dt/2) / hbar)
+  FxRec* Sfx[2];       // complex128: the same in fixed point, and V_s
+  double* Vs;
 };
 
 // <psi|A|psi> partial sums per block (k_expect_partial) and their fixed-order total.

@@ -1726,6 +1726,12 @@ __global__ void __launch_bounds__(256) k_static_phase(const StaticPhaseParams<T>
     p.S[0][i] = make_rec<T>(cs, sn);
     sincos(-V * (0.5 * p.g.dt) / p.g.hbar, &sn, &cs);
     p.S[1][i] = make_rec<T>(cs, sn);
+    if constexpr (std::is_same<T, double>::value) {
+      p.Sfx[1][i] = fx_rec_of(cs, sn);
+      sincos(-V * p.g.dt / p.g.hbar, &sn, &cs);
+      p.Sfx[0][i] = fx_rec_of(cs, sn);
+      p.Vs[i] = V;
+    }
   }
 }
 

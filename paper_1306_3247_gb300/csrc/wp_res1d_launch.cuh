@@ -2,7 +2,7 @@
 // threads), shared by the per-precision translation units wp_res1d_*.cu.
 #pragma once
 
-#include "wp_kernels.cuh"
+#include "wp_res1d_fx.cuh"
 
 namespace wp {
 namespace res1d_detail {
@@ -13,9 +13,14 @@ constexpr bool supported() {
   return sizeof(cx<T>) == 8 || LOGN <= 13;
 }
 
+// complex128 lines run in fixed point
 template <class T, int LOGN>
 cudaError_t launch_n(const Res1dParams<T>& p, size_t smem, cudaStream_t st) {
-  if constexpr (supported<T, LOGN>()) {
+  if constexpr (std::is_same<T, double>::value && supported<T, LOGN>()) {
+    using SH = r1fx::Shape<LOGN>;
+    r1fx::k_res1d_fx<LOGN><<<1, SH::NT + SH::TW, SH::SMEM, st>>>(p);
+    return cudaGetLastError();
+  } else if constexpr (supported<T, LOGN>()) {
     constexpr int EPT = wp_res1d_fixed_ept(LOGN);
     k_res1d_fixed<T, LOGN, EPT><<<1, (1 << LOGN) / EPT, smem, st>>>(p);
     return cudaGetLastError();
@@ -25,7 +30,11 @@ cudaError_t launch_n(const Res1dParams<T>& p, size_t smem, cudaStream_t st) {
 
 template <class T, int LOGN>
 cudaError_t launch_batch_n(const Res1dParams<T>* params, int ninst, int64_t nsteps, size_t smem, cudaStream_t st) {
-  if constexpr (supported<T, LOGN>()) {
+  if constexpr (std::is_same<T, double>::value && supported<T, LOGN>()) {
+    using SH = r1fx::Shape<LOGN>;
+    r1fx::k_res1d_fx_batch<LOGN><<<(unsigned)ninst, SH::NT + SH::TW, SH::SMEM, st>>>(params, nsteps);
+    return cudaGetLastError();
+  } else if constexpr (supported<T, LOGN>()) {
     constexpr int EPT = wp_res1d_fixed_ept(LOGN);
     k_res1d_fixed_batch<T, LOGN, EPT><<<(unsigned)ninst, (1 << LOGN) / EPT, smem, st>>>(params, nsteps);
     return cudaGetLastError();
@@ -35,7 +44,13 @@ cudaError_t launch_batch_n(const Res1dParams<T>* params, int ninst, int64_t nste
 
 template <class T, int LOGN>
 cudaError_t set_limit(int smem) {
-  if constexpr (supported<T, LOGN>()) {
+  if constexpr (std::is_same<T, double>::value && supported<T, LOGN>()) {
+    const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    const int need = (int)r1fx::Shape<LOGN>::SMEM;
+    cudaError_t e = cudaFuncSetAttribute(r1fx::k_res1d_fx<LOGN>, a, need);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(r1fx::k_res1d_fx_batch<LOGN>, a, need);
+    return e;
+  } else if constexpr (supported<T, LOGN>()) {
     constexpr int EPT = wp_res1d_fixed_ept(LOGN);
     const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
     cudaError_t e = cudaFuncSetAttribute(k_res1d_fixed<T, LOGN, EPT>, a, smem);
