@@ -87,10 +87,10 @@ struct wp_handle {
   int res_ept = 8;
   int res_max_radix_log = 3;
   size_t res_smem = 0;
-  bool res_fixed = false;          // 1-D line of compile-time length (k_res1d_fixed)
+  bool res_fixed = false;          // 1-D line of compile-time length (wp_line.cuh)
   void* res_S = nullptr;           // 1-D static phase tables, 2 x n records (dt, dt/2)
-  FxRec* res_Sfx = nullptr;        // complex128: the same in fixed point,
-  double* res_Vs = nullptr;        // and the static potential
+  FxRec* res_Sfx = nullptr;        // complex128: the same in fixed point
+  double* res_Vs = nullptr;        // 1-D static potential
   void* gauss_tab = nullptr;       // per-axis factors of the initial Gaussian
   double* vgrid = nullptr;         // static grid potential (FP64, N values), or NULL
   void* vgrid_rec[2] = {nullptr, nullptr};  // its phase records for dt, dt/2 (2-D, 3-D)
@@ -342,6 +342,7 @@ wp_status alloc_tables(wp_handle* h) {
   size_t off_w256[3] = {0, 0, 0};
   size_t off_w2s[3] = {0, 0, 0};
   size_t off_fx[3][4] = {};
+  size_t off_ln = 0;
   for (int d = 0; d < h->ndim; d++) {
     const size_t n = (size_t)h->n[d];
     for (int k = 0; k < 4; k++) off[d][k] = add(n * sizeof(cx<T>));
@@ -361,6 +362,7 @@ wp_status alloc_tables(wp_handle* h) {
     off_w2s[d] = (std::is_same<T, float>::value && (n == 64 || n == 128)) ? add(256 * 16) : 0;
     if (std::is_same<T, double>::value)
       for (int k = 0; k < 4; k++) off_fx[d][k] = add(n * sizeof(FxRec));
+    if (h->ndim == 1) off_ln = add(n * (std::is_same<T, double>::value ? sizeof(FxRec) : 16));
   }
   WP_CUDA(h, dev_malloc(h, &h->tabmem, bytes));
   WP_CUDA(h, cudaMemsetAsync(h->tabmem, 0, bytes, h->stream));
@@ -395,6 +397,7 @@ wp_status alloc_tables(wp_handle* h) {
       tb[d].Kfx_half = (FxRec*)(base + off_fx[d][2]);
       tb[d].Pfx = (FxRec*)(base + off_fx[d][3]);
     }
+    tb[d].Wln = h->ndim == 1 ? (void*)(base + off_ln) : nullptr;
   }
   // static tables (high and low parts)
   for (int d = 0; d < h->ndim; d++) {
@@ -452,6 +455,18 @@ wp_status alloc_tables(wp_handle* h) {
       }
       WP_CUDA(h, cudaMemcpy(tb[d].Wst, rec.data(), rec.size(), cudaMemcpyHostToDevice));
       if (!fx.empty()) WP_CUDA(h, cudaMemcpy(tb[d].Wfx, fx.data(), n * sizeof(FxRec), cudaMemcpyHostToDevice));
+      if (tb[d].Wln) {
+        const size_t rb = fx.empty() ? 16 : sizeof(FxRec);
+        const unsigned char* from = fx.empty() ? rec.data() : (const unsigned char*)fx.data();
+        std::vector<unsigned char> ln(n * rb, 0);
+        for (int l = 0; l < logn; l += wp_stage_radix_log(logn, l)) {
+          const int off = wp_stage_tw_offset(logn, l), rx = (1 << wp_stage_radix_log(logn, l)) - 1;
+          for (int jm = 0; l > 0 && jm < (1 << l); jm++)
+            for (int r = 0; r < rx; r++)
+              memcpy(&ln[((size_t)off + (size_t)r * (1 << l) + jm) * rb], from + ((size_t)off + (size_t)jm * rx + r) * rb, rb);
+        }
+        WP_CUDA(h, cudaMemcpy(tb[d].Wln, ln.data(), ln.size(), cudaMemcpyHostToDevice));
+      }
     }
     if (tb[d].W256) {
       // two-stage 256-point kernels: exp(-2 pi i t k1/256) at k1 * 16 + t (complex64: high +
@@ -735,7 +750,7 @@ wp_status apply_schedule(wp_handle* h, const wp_schedule& sc) {
     const int64_t n = h->n[0];
     const int ln = h->g.ln[0];
     const bool fx = sc.fixed && ln >= kRes1dLogMin && ln <= (h->elem == 8 ? kRes1dLogMax : 13);
-    const int E = fx ? wp_res1d_fixed_ept(ln) : ((n > 2048 || sc.ept >= 16) ? 16 : 8);
+    const int E = fx ? 8 : ((n > 2048 || sc.ept >= 16) ? 16 : 8);
     const int64_t thr = std::max<int64_t>(1, n / E);
     const int nthr = (int)((thr + 31) / 32 * 32);
     const bool ok = fx || (E == 8 && nthr <= 256) || (E == 16 && nthr <= 1024);
@@ -822,7 +837,7 @@ Res1dParams<T> res1d_params(wp_handle* h) {
   p.Wst = tb[0].Wst;
   p.Krec[0] = tb[0].Kfull_rec;
   p.Krec[1] = tb[0].Khalf_rec;
-  p.Wfx = tb[0].Wfx;
+  p.Wln = tb[0].Wln;
   p.Kfx[0] = tb[0].Kfx_full;
   p.Kfx[1] = tb[0].Kfx_half;
   p.Sfx[0] = h->res_Sfx;
@@ -1751,11 +1766,11 @@ wp_status wp_create_pooled(const wp_problem* pb, void* stream, void* mem_pool, w
   if (h->ndim == 1) {
     if ((e = dev_malloc(h, &h->res_S, 2 * (size_t)h->n[0] * sizeof(TwE<double>))) != cudaSuccess)
       return bail(cuda_fail(h, e, "static phase allocation"));
-    if (h->prec == WP_C128) {
-      if ((e = dev_malloc(h, (void**)&h->res_Sfx, 2 * (size_t)h->n[0] * sizeof(FxRec))) != cudaSuccess ||
-          (e = dev_malloc(h, (void**)&h->res_Vs, (size_t)h->n[0] * sizeof(double))) != cudaSuccess)
+    if ((e = dev_malloc(h, (void**)&h->res_Vs, (size_t)h->n[0] * sizeof(double))) != cudaSuccess)
+      return bail(cuda_fail(h, e, "static phase allocation"));
+    if (h->prec == WP_C128)
+      if ((e = dev_malloc(h, (void**)&h->res_Sfx, 2 * (size_t)h->n[0] * sizeof(FxRec))) != cudaSuccess)
         return bail(cuda_fail(h, e, "static phase allocation"));
-    }
     if ((st = res1d_split_potential(h)) != WP_OK) return bail(st);
   }
   if ((st = ensure_obs(h, 64)) != WP_OK) return bail(st);

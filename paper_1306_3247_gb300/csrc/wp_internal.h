@@ -61,8 +61,6 @@ __host__ __device__ constexpr int wp_stage_tw_offset(int logn, int logNs) {
 }
 constexpr int kFixedLogMin = 6, kFixedLogMax = 10;  // fixed-size pass kernels: n = 64..1024
 constexpr int kRes1dLogMin = 8, kRes1dLogMax = 14;  // fixed-length resident lines: n = 256..16384
-// elements per thread of a fixed-length resident line (1024 threads at most)
-__host__ __device__ constexpr int wp_res1d_fixed_ept(int logn) { return logn >= 14 ? 16 : 8; }
 
 // A table factor as one 16-byte record: the value for FP64 and float-float, the high
 // and low FP32 parts for the complex64 form.
@@ -176,6 +174,9 @@ struct AxisTab {
   FxRec* Kfx_full;
   FxRec* Kfx_half;
   FxRec* Pfx;
+  // 1-D lines: the stage twiddles with r outermost (twiddle r of index jm at (r - 1) Ns + jm
+  // of its stage), which neighbouring threads read side by side
+  void* Wln;
 };
 
 template <class T>
@@ -291,16 +292,15 @@ struct Res1dParams {
   uint32_t plane_mask;
   uint32_t gen_mask;
   const double* vgrid;       // static grid potential (observables; the phase is in S), or NULL
-  int32_t fixed;             // compile-time line length (k_res1d_fixed), n = 2^8 .. 2^14
+  int32_t fixed;             // compile-time line length (wp_line.cuh), n = 2^8 .. 2^14
   int32_t max_radix_log;     // largest butterfly of the run-time-length kernel (2 or 3)
   const void* Wst;           // per-stage twiddle records (fixed)
   const TwE<T>* Krec[2];     // kinetic factors dt, dt/2 as records (fixed)
-  // complex128 (fixed, wp_res1d_fx.cuh): fixed-point twiddles, kinetic factors without 1/n
-  // and static phases (dt, dt/2), and the static potential itself (observables)
-  const FxRec* Wfx;
+  const void* Wln;           // stage twiddles (fixed): records of the form, FxRec for complex128
+  // complex128 (fixed): kinetic factors without 1/n and static phases (dt, dt/2) in fixed point
   const FxRec* Kfx[2];
   const FxRec* Sfx[2];
-  const double* Vs;
+  const double* Vs;          // static potential (observables)
 };
 
 // Static phase tables of a 1-D handle (k_static_phase), formed in FP64 and stored as records.
@@ -312,8 +312,8 @@ struct StaticPhaseParams {
   uint32_t static_mask;
   const double* vgrid; // static grid potential added to V_s, or NULL
   TwE<T>* S[2];        // exp(-i V_s dt / hbar), exp(-i V_s (dt/2) / hbar)
-  FxRec* Sfx[2];       // complex128: the same in fixed point, and V_s
-  double* Vs;
+  FxRec* Sfx[2];       // complex128: the same in fixed point
+  double* Vs;          // V_s
 };
 
 // <psi|A|psi> partial sums per block (k_expect_partial) and their fixed-order total.

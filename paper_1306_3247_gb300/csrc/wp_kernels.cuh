@@ -1493,31 +1493,17 @@ __global__ void __launch_bounds__(256) k_prep_batch(const PrepParams<T>* __restr
 // evaluated at every point in FP64. The factors are applied one after the other as
 // records (complex64: high and low parts), so that the per-point work of the common
 // potentials stays off the FP64 pipe.
-// Line shape of the resident kernel: Res1dDyn holds the length and block size at run
-// time (E elements per thread, run-time Stockham stages); Res1dFix<LOGN, EPT> makes them
-// compile-time constants (n = 2^LOGN, n / EPT threads, unrolled stages with per-stage
-// twiddle records, kinetic factors as records).
+// This kernel takes any length (Res1dDyn: length and block size at run time, E elements per
+// thread, run-time Stockham stages); lines of 2^8 .. 2^14 points under the fixed schedule run
+// wp_line.cuh.
 template <int E>
 struct Res1dDyn {
-  static constexpr bool fixed = false;
   int logn, n, nthr;
   template <class T>
   __device__ explicit Res1dDyn(const Res1dParams<T>& p) : logn(p.logn), n(1 << p.logn), nthr(p.nthreads) {}
   template <class T, bool INV>
   __device__ __forceinline__ void fft(cx<T>* s, const Res1dParams<T>& p, int tid) const {
     fft_tile<T, E, INV>(s, logn, 0, 1, p.W, p.W_lo, tid, nthr, p.max_radix_log);
-  }
-};
-
-template <int LOGN, int EPT>
-struct Res1dFix {
-  static constexpr bool fixed = true;
-  static constexpr int logn = LOGN, n = 1 << LOGN, nthr = (1 << LOGN) / EPT;
-  template <class T>
-  __device__ explicit Res1dFix(const Res1dParams<T>&) {}
-  template <class T, bool INV>
-  __device__ __forceinline__ void fft(cx<T>* s, const Res1dParams<T>& p, int tid) const {
-    fft_fixed<T, LOGN, 0, 1, INV, 0, EPT, false>(s, reinterpret_cast<const TwE<T>*>(p.Wst), tid);
   }
 };
 
@@ -1588,16 +1574,10 @@ __device__ void res1d_potential_phase(cx<T>* s, const Res1dParams<T>& p, const R
 template <class T, class RS>
 __device__ void res1d_kinetic(cx<T>* s, const Res1dParams<T>& p, const RS& rs, int half, int tid) {
   rs.template fft<T, false>(s, p, tid);
-  if constexpr (RS::fixed) {
-    const TwE<T>* K = p.Krec[half];
-#pragma unroll
-    for (int i = tid; i < rs.n; i += rs.nthr) s[i] = tw_apply<false>(s[i], K[i]);
-  } else {
-    const cx<T>* K = half ? p.Khalf : p.Kfull;
-    const cx<T>* Klo = half ? p.Khalf_lo : p.Kfull_lo;
-    const cx<T> one = mk((T)1, (T)0), zero = mk((T)0, (T)0);
-    for (int i = tid; i < rs.n; i += rs.nthr) s[i] = apply_factor(s[i], K[i], Klo[i], one, zero);
-  }
+  const cx<T>* K = half ? p.Khalf : p.Kfull;
+  const cx<T>* Klo = half ? p.Khalf_lo : p.Kfull_lo;
+  const cx<T> one = mk((T)1, (T)0), zero = mk((T)0, (T)0);
+  for (int i = tid; i < rs.n; i += rs.nthr) s[i] = apply_factor(s[i], K[i], Klo[i], one, zero);
   __syncthreads();
   rs.template fft<T, true>(s, p, tid);
 }
@@ -1698,13 +1678,6 @@ __global__ void __launch_bounds__(MAXT) k_res1d(const Res1dParams<T> p) {
   res1d_body<T>(p, Res1dDyn<E>(p), reinterpret_cast<cx<T>*>(smem_raw));
 }
 
-// Fixed-length resident line: n = 2^LOGN, n / EPT threads.
-template <class T, int LOGN, int EPT>
-__global__ void __launch_bounds__((1 << LOGN) / EPT) k_res1d_fixed(const Res1dParams<T> p) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  res1d_body<T>(p, Res1dFix<LOGN, EPT>(p), reinterpret_cast<cx<T>*>(smem_raw));
-}
-
 // Static phase tables: exp(-i V_s(x_j) tau / hbar) for tau = dt and dt/2, V_s the sum of
 // the static terms (time-independent coefficient and centre) of a 1-D potential, formed
 // in FP64 and stored as records of T.
@@ -1726,11 +1699,11 @@ __global__ void __launch_bounds__(256) k_static_phase(const StaticPhaseParams<T>
     p.S[0][i] = make_rec<T>(cs, sn);
     sincos(-V * (0.5 * p.g.dt) / p.g.hbar, &sn, &cs);
     p.S[1][i] = make_rec<T>(cs, sn);
+    p.Vs[i] = V;
     if constexpr (std::is_same<T, double>::value) {
       p.Sfx[1][i] = fx_rec_of(cs, sn);
       sincos(-V * p.g.dt / p.g.hbar, &sn, &cs);
       p.Sfx[0][i] = fx_rec_of(cs, sn);
-      p.Vs[i] = V;
     }
   }
 }
@@ -1803,13 +1776,6 @@ template <class T, int E, int MAXT>
 __global__ void __launch_bounds__(MAXT) k_res1d_batch(const Res1dParams<T>* __restrict__ params, int64_t nsteps) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   res1d_batch_body<T, Res1dDyn<E>>(params, nsteps, reinterpret_cast<cx<T>*>(smem_raw));
-}
-
-template <class T, int LOGN, int EPT>
-__global__ void __launch_bounds__((1 << LOGN) / EPT)
-    k_res1d_fixed_batch(const Res1dParams<T>* __restrict__ params, int64_t nsteps) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  res1d_batch_body<T, Res1dFix<LOGN, EPT>>(params, nsteps, reinterpret_cast<cx<T>*>(smem_raw));
 }
 
 #ifdef WP_COMMON_KERNELS

@@ -1,8 +1,8 @@
-// Host launchers of the fixed-length resident-line kernels (n = 2^8 .. 2^14, n / EPT
-// threads), shared by the per-precision translation units wp_res1d_*.cu.
+// Host launchers of the resident lines of compile-time length (n = 2^8 .. 2^14, wp_line.cuh),
+// shared by the per-precision translation units wp_res1d_*.cu.
 #pragma once
 
-#include "wp_res1d_fx.cuh"
+#include "wp_line.cuh"
 
 namespace wp {
 namespace res1d_detail {
@@ -13,48 +13,67 @@ constexpr bool supported() {
   return sizeof(cx<T>) == 8 || LOGN <= 13;
 }
 
-// complex128 lines run in fixed point
+// Blocks (log2) of the cluster that holds a line, alone and as one of a batch. Alone, a line
+// takes eight SMs (the portable cluster) as soon as each block has two warps of points:
+// complex128 at 4096 points 27.8 us per step on one block, 11.0 on eight. At 1024 points one
+// warp per block would be left, with nothing gained over four warps of one block. In a batch
+// the lines fill the GPU by themselves and a cluster only adds exchanges (256 lines of the
+// uneven batch beside its 2-D passes: 2.07 ms per 20 steps with clusters of four and eight
+// for 2048 points and more, 1.66 without), so that only lines of more points than 512
+// threads hold are split.
+template <int LOGN>
+constexpr int cluster_log() {
+  return LOGN <= 10 ? 0 : (LOGN == 11 ? 2 : 3);
+}
+template <int LOGN>
+constexpr int batch_cluster_log() {
+  return LOGN <= 12 ? 0 : LOGN - 12;
+}
+
+template <class SH, class K, class... A>
+cudaError_t go(K kern, unsigned nlines, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(nlines * SH::R);
+  cfg.blockDim = dim3(SH::NT + SH::TW);
+  cfg.dynamicSmemBytes = SH::SMEM;
+  cfg.stream = st;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = SH::R;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = SH::R > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 template <class T, int LOGN>
-cudaError_t launch_n(const Res1dParams<T>& p, size_t smem, cudaStream_t st) {
-  if constexpr (std::is_same<T, double>::value && supported<T, LOGN>()) {
-    using SH = r1fx::Shape<LOGN>;
-    r1fx::k_res1d_fx<LOGN><<<1, SH::NT + SH::TW, SH::SMEM, st>>>(p);
-    return cudaGetLastError();
-  } else if constexpr (supported<T, LOGN>()) {
-    constexpr int EPT = wp_res1d_fixed_ept(LOGN);
-    k_res1d_fixed<T, LOGN, EPT><<<1, (1 << LOGN) / EPT, smem, st>>>(p);
-    return cudaGetLastError();
+cudaError_t launch_n(const Res1dParams<T>& p, size_t, cudaStream_t st) {
+  if constexpr (supported<T, LOGN>()) {
+    constexpr int LOGR = cluster_log<LOGN>();
+    using SH = line::Shape<T, LOGN, LOGR>;
+    return go<SH>(line::k_line<T, LOGN, LOGR>, 1, st, p);
   }
   return cudaErrorInvalidConfiguration;
 }
 
 template <class T, int LOGN>
-cudaError_t launch_batch_n(const Res1dParams<T>* params, int ninst, int64_t nsteps, size_t smem, cudaStream_t st) {
-  if constexpr (std::is_same<T, double>::value && supported<T, LOGN>()) {
-    using SH = r1fx::Shape<LOGN>;
-    r1fx::k_res1d_fx_batch<LOGN><<<(unsigned)ninst, SH::NT + SH::TW, SH::SMEM, st>>>(params, nsteps);
-    return cudaGetLastError();
-  } else if constexpr (supported<T, LOGN>()) {
-    constexpr int EPT = wp_res1d_fixed_ept(LOGN);
-    k_res1d_fixed_batch<T, LOGN, EPT><<<(unsigned)ninst, (1 << LOGN) / EPT, smem, st>>>(params, nsteps);
-    return cudaGetLastError();
+cudaError_t launch_batch_n(const Res1dParams<T>* params, int ninst, int64_t nsteps, size_t, cudaStream_t st) {
+  if constexpr (supported<T, LOGN>()) {
+    constexpr int LOGR = batch_cluster_log<LOGN>();
+    using SH = line::Shape<T, LOGN, LOGR, true>;
+    return go<SH>(line::k_line_batch<T, LOGN, LOGR>, (unsigned)ninst, st, params, nsteps);
   }
   return cudaErrorInvalidConfiguration;
 }
 
 template <class T, int LOGN>
-cudaError_t set_limit(int smem) {
-  if constexpr (std::is_same<T, double>::value && supported<T, LOGN>()) {
+cudaError_t set_limit(int) {
+  if constexpr (supported<T, LOGN>()) {
+    constexpr int LOGR = cluster_log<LOGN>(), LOGB = batch_cluster_log<LOGN>();
     const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    const int need = (int)r1fx::Shape<LOGN>::SMEM;
-    cudaError_t e = cudaFuncSetAttribute(r1fx::k_res1d_fx<LOGN>, a, need);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(r1fx::k_res1d_fx_batch<LOGN>, a, need);
-    return e;
-  } else if constexpr (supported<T, LOGN>()) {
-    constexpr int EPT = wp_res1d_fixed_ept(LOGN);
-    const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    cudaError_t e = cudaFuncSetAttribute(k_res1d_fixed<T, LOGN, EPT>, a, smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_res1d_fixed_batch<T, LOGN, EPT>, a, smem);
+    cudaError_t e = cudaFuncSetAttribute(line::k_line<T, LOGN, LOGR>, a, (int)line::Shape<T, LOGN, LOGR>::SMEM);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(line::k_line_batch<T, LOGN, LOGB>, a, (int)line::Shape<T, LOGN, LOGB, true>::SMEM);
     return e;
   }
   return cudaSuccess;
