@@ -519,14 +519,14 @@ wp_status alloc_tables(wp_handle* h) {
     host_kinetic(h, d, h->pb.dt, scale, re, im, pfx);
     split();
     if (pfx) WP_CUDA(h, cudaMemcpy(tb[d].Kfx_full, fx.data(), n * sizeof(FxRec), cudaMemcpyHostToDevice));
-    for (size_t k = 0; k < n; k++) recs[k] = make_rec<T>(re[k], im[k]);
+    for (size_t k = 0; k < n; k++) recs[k] = h->ndim > 1 ? make_axis_rec<T>(re[k], im[k], scale) : make_rec<T>(re[k], im[k]);
     WP_CUDA(h, cudaMemcpy(tb[d].Kfull, hi.data(), nb, cudaMemcpyHostToDevice));
     WP_CUDA(h, cudaMemcpy(tb[d].Kfull_lo, lo.data(), nb, cudaMemcpyHostToDevice));
     WP_CUDA(h, cudaMemcpy(tb[d].Kfull_rec, recs.data(), n * sizeof(TwE<T>), cudaMemcpyHostToDevice));
     host_kinetic(h, d, 0.5 * h->pb.dt, scale, re, im, pfx);
     split();
     if (pfx) WP_CUDA(h, cudaMemcpy(tb[d].Kfx_half, fx.data(), n * sizeof(FxRec), cudaMemcpyHostToDevice));
-    for (size_t k = 0; k < n; k++) recs[k] = make_rec<T>(re[k], im[k]);
+    for (size_t k = 0; k < n; k++) recs[k] = h->ndim > 1 ? make_axis_rec<T>(re[k], im[k], scale) : make_rec<T>(re[k], im[k]);
     WP_CUDA(h, cudaMemcpy(tb[d].Khalf, hi.data(), nb, cudaMemcpyHostToDevice));
     WP_CUDA(h, cudaMemcpy(tb[d].Khalf_lo, lo.data(), nb, cudaMemcpyHostToDevice));
     WP_CUDA(h, cudaMemcpy(tb[d].Khalf_rec, recs.data(), n * sizeof(TwE<T>), cudaMemcpyHostToDevice));

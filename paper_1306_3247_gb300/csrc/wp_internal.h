@@ -1,6 +1,7 @@
 // Internal host/device declarations of the split-operator library.
 #pragma once
 
+#include <cmath>
 #include <cstdint>
 
 #include "wavepacket_gpu.h"
@@ -87,6 +88,35 @@ __host__ __device__ inline TwE<float> make_rec<float>(double re, double im) {
   r.h = cx<float>{hr, hi};
   r.l = cx<float>{(float)(re - (double)hr), (float)(im - (double)hi)};
   return r;
+}
+
+// Records of factors that are applied as products of an axis record and a line record. For
+// complex64 the high parts are multiples of 2^-11 (axis) and 2^-12 (line), the low parts the
+// rest (36 bits in all), so that the product of two high parts is exact in FP32
+// (mul_line_axis). scale: a power of two that the factor carries.
+template <class T>
+__host__ __device__ inline TwE<T> make_axis_rec(double re, double im, double scale = 1.0) {
+  (void)scale;
+  return make_rec<T>(re, im);
+}
+template <class T>
+__host__ __device__ inline TwE<T> make_line_rec(double re, double im) {
+  return make_rec<T>(re, im);
+}
+__host__ __device__ inline TwE<float> make_grid_rec(double re, double im, double unit) {
+  TwE<float> r;
+  const double gr = rint(re / unit) * unit, gi = rint(im / unit) * unit;
+  r.h = cx<float>{(float)gr, (float)gi};
+  r.l = cx<float>{(float)(re - gr), (float)(im - gi)};
+  return r;
+}
+template <>
+__host__ __device__ inline TwE<float> make_axis_rec<float>(double re, double im, double scale) {
+  return make_grid_rec(re, im, scale * 0x1p-11);
+}
+template <>
+__host__ __device__ inline TwE<float> make_line_rec<float>(double re, double im) {
+  return make_grid_rec(re, im, 0x1p-12);
 }
 
 // A unit factor c + i s of the fixed-point transforms (wp_fx.h): c, c + s and c - s times

@@ -193,14 +193,14 @@ __device__ __forceinline__ ff table_value(const ff* p) { return *p; }
 // Gaussian terms skip whole lines whose coefficient is negligible (gauss_line_active).
 
 // A factor that is the product of a line factor L (the other axes) and an axis factor a:
-// complex64 forms the product a L exactly (error-free products and sums of the high + low
-// parts) and rounds v a L once. Two roundings (v L, then (v L) a) drift the norm of a
+// complex64 forms the product a L to about 2^-35 from high parts on grids that make their
+// products exact (apply_factor_rec) and rounds v a L once. Two roundings (v L, then (v L) a) drift the norm of a
 // nearly periodic state by about 1e-8 per step: its points repeat, and so do their
 // rounding errors (measured: 1.3e-5 after 1000 steps of the 128^2 trapped packet, against
 // 1e-6 with one rounding). Float-float applies the two records one after the other
 // (error-free complex products, about 48 bits).
 __device__ __forceinline__ cx<float> mul_line_axis(cx<float> v, const TwE<float>& L, const TwE<float>& a) {
-  return apply_factor(v, a.h, a.l, L.h, L.l);
+  return apply_factor_rec(v, a, L);
 }
 __device__ __forceinline__ cx<ff> mul_line_axis(cx<ff> v, const TwE<ff>& L, const TwE<ff>& a) {
   return tw_apply<false>(tw_apply<false>(v, L), a);
