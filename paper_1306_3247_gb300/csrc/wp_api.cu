@@ -611,25 +611,6 @@ PassParams<T> pass_params(wp_handle* h, int axis, uint32_t flags, void* in, void
   return p;
 }
 
-template <class T>
-LinesParams<T> phase_lines_params(wp_handle* h) {
-  LinesParams<T> p{};
-  AxisTab<T>* tb = tabs<T>(h);
-  p.g = h->g;
-  p.axis = h->ndim - 1;
-  p.gauss = 1;
-  p.ngauss = h->hpot.ngauss;
-  p.nlines = h->nlines_phase;
-  for (int d = 0; d < h->ndim; d++) {
-    p.H[d] = tb[d].P;
-    p.Lo[d] = tb[d].P_lo;
-    for (int gg = 0; gg < WP_MAX_GAUSS; gg++) p.Gd[gg][d] = tb[d].Gd[gg];
-  }
-  p.ctrl = h->ctrl;
-  p.out = (LineRec<T>*)h->lines_phase;
-  return p;
-}
-
 // Per-line records of the contiguous (potential) or kinetic pass.
 template <class T>
 wp_status run_lines(wp_handle* h, bool phase, int khalf) {
@@ -684,14 +665,16 @@ wp_status run_prep(wp_handle* h, int step_add, double t_shift, double tau, bool 
   p.ctrl = h->ctrl;
   p.step_add = step_add;
   p.t_shift = t_shift;
-  p.tau = tau;
+  p.tau_dt = tau == h->pb.dt ? 1.0 : tau / h->pb.dt;
+  p.dt_hbar = h->pb.dt / h->pb.hbar;
+  p.lines = phase_lines && h->ndim == 2 ? (LineRec<T>*)h->lines_phase : nullptr;
   h->phase_half = tau == h->pb.dt ? 0 : (tau == 0.5 * h->pb.dt ? 1 : -1);
   {
     LaunchScope ls(h, K_PREP);
-    wp_status st = launch_rc(h, launch_prep<T>(p, h->stream), "prep kernel");
+    wp_status st = launch_rc(h, launch_prep<T>(p, h->hpot.ngauss, h->stream), "prep kernel");
     if (st != WP_OK) return st;
   }
-  if (phase_lines && h->ndim > 1) return run_lines<T>(h, true, 0);
+  if (phase_lines && h->ndim > 2) return run_lines<T>(h, true, 0);
   return WP_OK;
 }
 
@@ -927,7 +910,6 @@ wp_status momentum_and_reduce(wp_handle* h) {
   r.mom = h->part_mom;
   r.nmom = h->rows_mom;
   r.g = h->g;
-  r.ntotal = h->N;
   r.autocorr = h->pb.autocorr ? 1 : 0;
   r.ctrl = h->ctrl;
   r.obs_out = h->obs_dev;
@@ -1252,8 +1234,6 @@ struct wp_batch {
   void* d_pass_z = nullptr;
   void* d_pass_x = nullptr;
   void* d_prep = nullptr;
-  void* d_lines = nullptr;
-  int64_t max_lines = 0;
   int64_t* d_tiles_z = nullptr;
   int64_t* d_tiles_x = nullptr;
   int* d_binst_z = nullptr;   // instance of every block of the batched passes
@@ -1284,13 +1264,12 @@ void batch_free_compiled(wp_batch* b) {
   for (auto& kv : b->graphs) cudaGraphExecDestroy(kv.second);
   b->graphs.clear();
   b->seen.clear();
-  void* ps[] = {b->d_pass_z, b->d_pass_x, b->d_prep, b->d_lines, b->d_tiles_z, b->d_tiles_x, b->d_binst_z,
+  void* ps[] = {b->d_pass_z, b->d_pass_x, b->d_prep, b->d_tiles_z, b->d_tiles_x, b->d_binst_z,
                 b->d_binst_x};
   for (void* q : ps)
     if (q) cudaFree(q);
-  b->d_pass_z = b->d_pass_x = b->d_prep = b->d_lines = nullptr;
+  b->d_pass_z = b->d_pass_x = b->d_prep = nullptr;
   b->d_binst_z = b->d_binst_x = nullptr;
-  b->max_lines = 0;
   b->d_tiles_z = b->d_tiles_x = nullptr;
   b->cls_z.clear();
   b->cls_x.clear();
@@ -1344,7 +1323,6 @@ wp_status batch_compile(wp_batch* b) {
   if (!b->idx2d.empty()) {
     std::vector<PassParams<T>> pz, px;
     std::vector<PrepParams<T>> pp;
-    std::vector<LinesParams<T>> pl;
     std::vector<int64_t> tz, tx;
     int64_t az = 0, ax = 0;
     for (int k : b->idx2d) {
@@ -1367,9 +1345,9 @@ wp_status batch_compile(wp_batch* b) {
       for (int d = 0; d < h->ndim; d++) q.tab[d] = tb[d];
       q.pot = h->dpot;
       q.ctrl = h->ctrl;
+      q.dt_hbar = h->pb.dt / h->pb.hbar;
+      q.lines = (LineRec<T>*)h->lines_phase;
       pp.push_back(q);
-      pl.push_back(phase_lines_params<T>(h));
-      b->max_lines = std::max(b->max_lines, h->nlines_phase);
       b->smem2d = std::max(b->smem2d, std::max(h->plan[0].smem, h->plan[1].smem));
     }
     b->ntiles_z = az;
@@ -1456,8 +1434,6 @@ wp_status batch_compile(wp_batch* b) {
     WP_CUDA(nullptr, cudaMalloc(&b->d_pass_z, pz.size() * sizeof(PassParams<T>)));
     WP_CUDA(nullptr, cudaMalloc(&b->d_pass_x, px.size() * sizeof(PassParams<T>)));
     WP_CUDA(nullptr, cudaMalloc(&b->d_prep, pp.size() * sizeof(PrepParams<T>)));
-    WP_CUDA(nullptr, cudaMalloc(&b->d_lines, pl.size() * sizeof(LinesParams<T>)));
-    WP_CUDA(nullptr, cudaMemcpy(b->d_lines, pl.data(), pl.size() * sizeof(LinesParams<T>), cudaMemcpyHostToDevice));
     WP_CUDA(nullptr, cudaMalloc(&b->d_tiles_z, tz.size() * sizeof(int64_t)));
     WP_CUDA(nullptr, cudaMalloc(&b->d_tiles_x, tx.size() * sizeof(int64_t)));
     WP_CUDA(nullptr, cudaMemcpy(b->d_pass_z, pz.data(), pz.size() * sizeof(PassParams<T>), cudaMemcpyHostToDevice));
@@ -1482,12 +1458,8 @@ wp_status batch_issue(wp_batch* b, int64_t m) {
   const int n2 = (int)b->idx2d.size();
   auto prep = [&](int add, double shift, double tau) -> wp_status {
     b->launches++;
-    wp_status r = launch_rc(nullptr, launch_prep_batch<T>((const PrepParams<T>*)b->d_prep, n2, add, shift, tau, st),
-                            "batched prep");
-    if (r != WP_OK || tau == 0.0) return r;
-    b->launches++;
-    return launch_rc(nullptr, launch_lines_batch<T>((const LinesParams<T>*)b->d_lines, n2, b->max_lines, st),
-                     "batched line records");
+    return launch_rc(nullptr, launch_prep_batch<T>((const PrepParams<T>*)b->d_prep, n2, add, shift, tau, st),
+                     "batched prep");
   };
   // One launch per pass over the merged classes (the kinetic one with the next step's
   // tables as leading blocks when asked: step increment, time shift, phase length in dt;
@@ -1498,8 +1470,7 @@ wp_status batch_issue(wp_batch* b, int64_t m) {
       const wp_status r = launch_rc(
           nullptr,
           launch_merged_contig<T>((const PassParams<T>*)b->d_pass_z, b->d_tiles_z, b->d_binst_z, b->ml_z, f, 0,
-                                  (const PrepParams<T>*)b->d_prep, (const LinesParams<T>*)b->d_lines,
-                                  b->smem_merged, st),
+                                  (const PrepParams<T>*)b->d_prep, b->smem_merged, st),
           "batched pass");
       if (r != WP_OK) return r;
     }
@@ -1520,15 +1491,13 @@ wp_status batch_issue(wp_batch* b, int64_t m) {
       ml.step_add = add;
       ml.shift_dt = shift;
       ml.tau_dt = tau;
-      ml.lines = tau != 0.0;
     }
     if (ml.ncls > 0 || ml.nprep > 0) {
       b->launches++;
       const wp_status r = launch_rc(
           nullptr,
           launch_merged_strided<T>((const PassParams<T>*)b->d_pass_x, b->d_tiles_x, b->d_binst_x, ml, F_KIN | FX, khalf,
-                                   (const PrepParams<T>*)b->d_prep, (const LinesParams<T>*)b->d_lines,
-                                   b->smem_merged, st),
+                                   (const PrepParams<T>*)b->d_prep, b->smem_merged, st),
           "batched pass");
       if (r != WP_OK) return r;
     }
@@ -1721,6 +1690,8 @@ wp_status wp_create_pooled(const wp_problem* pb, void* stream, void* mem_pool, w
   g.dt = pb->dt;
   g.t0 = pb->t0;
   h->N = h->n[0] * h->n[1] * h->n[2];
+  g.dvk = g.dv / (double)h->N;
+  g.ekin = g.hbar * g.hbar / (2.0 * g.mass);
   const size_t bytes = (size_t)h->N * h->elem;
   auto bail = [&](wp_status s) {
     g_err = h->err;

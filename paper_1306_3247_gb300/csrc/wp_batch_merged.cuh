@@ -1,7 +1,7 @@
 // One launch per pass of an uneven batch (the 2-D instances of wp_batch): the blocks of
 // the Stockham line-length classes of the pass run in the same grid, each block picking
 // its class from the launch's class table, and the per-instance tables and line records
-// of the next step (k_prep_batch and k_lines_batch work) run as leading blocks of the
+// of the next step (k_prep_batch's work) run as leading blocks of the
 // kinetic pass.
 // The kinetic pass reads neither the potential tables nor the line records of the
 // potential pass, and the potential pass that read the current ones has completed before
@@ -16,12 +16,10 @@
 
 namespace wp {
 
-// The per-instance tables of the step (prep_body with the instance's own parameters,
-// one block) followed, when `lines`, by the line records of its potential pass.
+// The per-instance tables and line records of the step (prep_body with the instance's own
+// parameters, one block).
 template <class T>
-__device__ __forceinline__ void prep_lines_block(const PrepParams<T>* __restrict__ pp,
-                                                 const LinesParams<T>* __restrict__ lp, int inst,
-                                                 const MergedLaunch& ml) {
+__device__ __forceinline__ void prep_block(const PrepParams<T>* __restrict__ pp, int inst, const MergedLaunch& ml) {
   __shared__ __align__(16) unsigned char raw[sizeof(PrepParams<T>)];
   PrepParams<T>& p = *reinterpret_cast<PrepParams<T>*>(raw);
   const int* src = reinterpret_cast<const int*>(&pp[inst]);
@@ -31,19 +29,11 @@ __device__ __forceinline__ void prep_lines_block(const PrepParams<T>* __restrict
   if (threadIdx.x == 0) {
     p.step_add = ml.step_add;
     p.t_shift = ml.shift_dt * p.g.dt;
-    p.tau = ml.tau_dt * p.g.dt;
+    p.tau_dt = ml.tau_dt;
+    if (ml.tau_dt == 0.0) p.lines = nullptr;
   }
   __syncthreads();
   prep_body<T>(p, 0, 1);
-  if (!ml.lines) return;
-  // the tables and the control block written above are visible to the whole block
-  __syncthreads();
-  __shared__ __align__(16) unsigned char rawl[sizeof(LinesParams<T>)];
-  const int* srcl = reinterpret_cast<const int*>(&lp[inst]);
-  for (int k = threadIdx.x; k < (int)(sizeof(LinesParams<T>) / sizeof(int)); k += blockDim.x)
-    reinterpret_cast<int*>(rawl)[k] = srcl[k];
-  __syncthreads();
-  lines_body<T>(*reinterpret_cast<const LinesParams<T>*>(rawl), threadIdx.x, blockDim.x);
 }
 
 // The two-stage complex64 body of a 64- (LOGT 3) or 128-point (LOGT 4) class.
@@ -121,9 +111,9 @@ template <class T, bool CONTIG>
 __global__ void __launch_bounds__(256, merged_min_blocks<T>())
     k_pass_batch_merged(const PassParams<T>* __restrict__ params, const int64_t* __restrict__ tile_start,
                         const int* __restrict__ block_inst, const MergedLaunch ml, uint32_t flags, int khalf,
-                        const PrepParams<T>* __restrict__ pp, const LinesParams<T>* __restrict__ lp) {
+                        const PrepParams<T>* __restrict__ pp) {
   if ((int64_t)blockIdx.x < ml.nprep) {
-    prep_lines_block<T>(pp, lp, (int)blockIdx.x, ml);
+    prep_block<T>(pp, (int)blockIdx.x, ml);
     return;
   }
   const int64_t b = (int64_t)blockIdx.x - ml.nprep;
@@ -137,8 +127,8 @@ __global__ void __launch_bounds__(256, merged_min_blocks<T>())
 // Host launcher (one translation unit per precision and pass kind).
 template <class T, bool CONTIG>
 int launch_merged(const PassParams<T>* params, const int64_t* tile_start, const int* block_inst,
-                  const MergedLaunch& ml, uint32_t flags, int khalf, const PrepParams<T>* pp,
-                  const LinesParams<T>* lp, size_t smem, void* stream) {
+                  const MergedLaunch& ml, uint32_t flags, int khalf, const PrepParams<T>* pp, size_t smem,
+                  void* stream) {
   static std::once_flag once;
   static cudaError_t attr = cudaSuccess;
   std::call_once(once, [] {
@@ -149,7 +139,7 @@ int launch_merged(const PassParams<T>* params, const int64_t* tile_start, const 
   const int64_t nblocks = ml.start[ml.ncls] + ml.nprep;
   if (nblocks > 0)
     k_pass_batch_merged<T, CONTIG><<<(unsigned)nblocks, 256, smem, (cudaStream_t)stream>>>(
-        params, tile_start, block_inst, ml, flags, khalf, pp, lp);
+        params, tile_start, block_inst, ml, flags, khalf, pp);
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? 0 : (int)e;
 }
@@ -160,8 +150,8 @@ int launch_merged(const PassParams<T>* params, const int64_t* tile_start, const 
   namespace wp {                                                                                                  \
   template <>                                                                                                     \
   int NAME<T>(const PassParams<T>* params, const int64_t* tile_start, const int* block_inst,                     \
-              const MergedLaunch& ml, uint32_t flags, int khalf, const PrepParams<T>* pp,                        \
-              const LinesParams<T>* lp, size_t smem, void* stream) {                                             \
-    return launch_merged<T, CONTIG>(params, tile_start, block_inst, ml, flags, khalf, pp, lp, smem, stream);     \
+              const MergedLaunch& ml, uint32_t flags, int khalf, const PrepParams<T>* pp, size_t smem,           \
+              void* stream) {                                                                                    \
+    return launch_merged<T, CONTIG>(params, tile_start, block_inst, ml, flags, khalf, pp, smem, stream);         \
   }                                                                                                               \
   }

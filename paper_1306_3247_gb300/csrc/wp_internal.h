@@ -163,6 +163,8 @@ struct Geom {
   double kscale[3];    // 2 pi / L
   double mass, hbar, dt, t0;
   double dv;           // cell volume
+  double dvk;          // dv / grid points
+  double ekin;         // hbar^2 / 2m
   // Powers of two at or above the largest |x_i| and |k_i| of each axis. The observable
   // tables of the line sums (Ox, Ok) hold x / oscale_x and k / oscale_k, so that sums
   // formed in FP32 range stay finite in any units (in SI units k^2 |psi_hat|^2 alone
@@ -288,7 +290,9 @@ struct PrepParams {
   Ctrl* ctrl;
   int32_t step_add;    // added to ctrl->step before the time is formed
   double t_shift;      // added to t0 + step dt (dt/2 for the mid-point order)
-  double tau;          // phase length (dt, dt/2 or 0 for observables only)
+  double tau_dt;       // phase length in units of dt (1, 1/2 or 0 for observables only)
+  double dt_hbar;      // dt / hbar
+  LineRec<T>* lines;   // 2-D: line records of the potential pass, or NULL
 };
 
 template <class T>
@@ -372,7 +376,6 @@ struct ReduceParams {
   int64_t nmom;
   int64_t pos_stride, mom_stride;
   Geom g;
-  int64_t ntotal;      // grid points
   int32_t autocorr;
   Ctrl* ctrl;
   double* obs_out;     // [cap][16]
@@ -400,7 +403,7 @@ struct GaussParams {
 
 // Launchers (defined per precision in the kernel translation units).
 template <class T> int launch_pass(const PassParams<T>& p, int64_t ntiles, size_t smem, void* stream);
-template <class T> int launch_prep(const PrepParams<T>& p, void* stream);
+template <class T> int launch_prep(const PrepParams<T>& p, int ngauss, void* stream);
 template <class T> int launch_res1d(const Res1dParams<T>& p, size_t smem, void* stream);
 template <class T> int launch_convert(const ConvParams<T>& p, void* stream);
 template <class T> int launch_gaussian(const GaussParams<T>& p, int64_t n, void* stream);
@@ -409,8 +412,6 @@ template <class T> int launch_lines(const LinesParams<T>& p, void* stream);
 template <class T> int launch_pass_batch(const PassParams<T>* params, const int64_t* tile_start, const int* block_inst,
                                          int logn, int64_t block_off, int64_t nblocks, uint32_t flags, int khalf,
                                          size_t smem, void* stream);
-template <class T> int launch_lines_batch(const LinesParams<T>* params, int ninst, int64_t max_lines,
-                                          void* stream);
 template <class T> int launch_prep_batch(const PrepParams<T>* params, int ninst, int step_add, double shift_dt,
                                          double tau_dt, void* stream);
 template <class T> int launch_res1d_batch(const Res1dParams<T>* params, int ninst, int nthreads, int ept,
@@ -431,8 +432,9 @@ template <class T> int launch_fixed(const PassParams<T>& p, unsigned ntiles, siz
 // One launch per batched pass (wp_batch_merged.cuh): class c of the pass covers launch
 // blocks start[c] .. start[c + 1] - 1 and block-list entries list_off[c] on; key[c] is its
 // line-length class (6..10 fixed-shape, kBatchClassP256 + v two-stage), counted after nprep
-// leading blocks that form the per-instance tables (and, with lines, the line records) of
-// the next step, with the step increment, time shift and phase length (units of dt) given.
+// leading blocks that form the per-instance tables (and, for a phase length other than 0, the
+// line records) of the next step, with the step increment, time shift and phase length (units
+// of dt) given.
 constexpr int kMergedMaxClasses = 8;
 struct MergedLaunch {
   int32_t ncls;
@@ -442,16 +444,15 @@ struct MergedLaunch {
   int32_t nprep;
   int32_t step_add;
   double shift_dt, tau_dt;
-  int32_t lines;
 };
 template <class T>
 int launch_merged_contig(const PassParams<T>* params, const int64_t* tile_start, const int* block_inst,
-                         const MergedLaunch& ml, uint32_t flags, int khalf, const PrepParams<T>* pp,
-                         const LinesParams<T>* lp, size_t smem, void* stream);
+                         const MergedLaunch& ml, uint32_t flags, int khalf, const PrepParams<T>* pp, size_t smem,
+                         void* stream);
 template <class T>
 int launch_merged_strided(const PassParams<T>* params, const int64_t* tile_start, const int* block_inst,
-                          const MergedLaunch& ml, uint32_t flags, int khalf, const PrepParams<T>* pp,
-                          const LinesParams<T>* lp, size_t smem, void* stream);
+                          const MergedLaunch& ml, uint32_t flags, int khalf, const PrepParams<T>* pp, size_t smem,
+                          void* stream);
 
 // two-stage kernels for 256-point lines, complex64 and float-float (wp_pass256_*.cu)
 template <class T> bool pass256_applies(const PassParams<T>& p);

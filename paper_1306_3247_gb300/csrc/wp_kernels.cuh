@@ -470,27 +470,44 @@ __device__ __forceinline__ void block_sum(double (&acc)[NQ], double* out, double
 
 // Observable record from the position sums qp and momentum sums qm (Tab. 3):
 // 0 t, 1 norm, 2-4 <x>, 5-7 <p>, 8-10 <x^2>, 11 E, 12 E_K, 13 E_V, 14 autocorrelation, 15 step.
-__device__ inline void finish_obs(const double* qp, const double* qm, const Geom& g, int64_t ntotal,
-                                  int autocorr, double t, int64_t step, double* rec) {
-  const double dv = g.dv;
-  const double dvk = dv / (double)ntotal;
-  rec[0] = t;
-  rec[1] = sqrt(qp[Q_RHO] * dv);
-  for (int d = 0; d < 3; d++) {
-    rec[2 + d] = qp[Q_X + d] * dv;
-    rec[5 + d] = g.hbar * qm[Q_K + d] * dvk;
-    rec[8 + d] = qp[Q_XX + d] * dv;
+// Called by the 32 lanes of a warp, each forming one entry (one thread alone took 3 us of FP64
+// latencies).
+__device__ __forceinline__ void finish_obs(const double* qp, const double* qm, const Geom& g, int autocorr, double t,
+                                           int64_t step, int lane, double* rec) {
+  double a = 0.0, b = 1.0;  // entry = a b
+  if (lane == 0) a = t;
+  if (lane == 15) a = (double)step;
+  if (lane == 1) a = qp[Q_RHO], b = g.dv;
+  if (lane >= 2 && lane < 5) a = qp[Q_X + lane - 2], b = g.dv;
+  if (lane >= 5 && lane < 8) a = qm[Q_K + lane - 5], b = g.hbar * g.dvk;
+  if (lane >= 8 && lane < 11) a = qp[Q_XX + lane - 8], b = g.dv;
+  if (lane == 11 || lane == 12) a = qm[Q_K2], b = g.ekin * g.dvk;
+  if (lane == 13) a = qp[Q_V], b = g.dv;
+  double v = a * b;
+  const double ev = __shfl_sync(0xffffffffu, v, 13);
+  if (lane == 11) v += ev;
+  if (lane == 1) v = sqrt(v);
+  if (lane == 14) v = autocorr ? (qp[Q_AC_RE] * qp[Q_AC_RE] + qp[Q_AC_IM] * qp[Q_AC_IM]) * g.dv * g.dv : 0.0;
+  if (lane < 16) rec[lane] = v;
+}
+
+// The record into the next slot of the run (the 32 lanes of one warp).
+__device__ __forceinline__ void publish_obs(const double* qp, const double* qm, const Geom& g, int autocorr, double t,
+                                            int64_t step, int lane, Ctrl* ctrl, double* obs_out, int64_t cap) {
+  const int64_t slot = ctrl->nobs;
+  __syncwarp();
+  if (slot < cap) {
+    double* rec = obs_out + slot * 16;
+    finish_obs(qp, qm, g, autocorr, t, step, lane, rec);
+    if (lane == 1 && !isfinite(rec[1])) ctrl->err = WP_ENONFINITE;
   }
-  rec[12] = g.hbar * g.hbar / (2.0 * g.mass) * qm[Q_K2] * dvk;
-  rec[13] = qp[Q_V] * dv;
-  rec[11] = rec[12] + rec[13];
-  rec[14] = autocorr ? (qp[Q_AC_RE] * qp[Q_AC_RE] + qp[Q_AC_IM] * qp[Q_AC_IM]) * dv * dv : 0.0;
-  rec[15] = (double)step;
+  if (lane == 0) ctrl->nobs = slot + 1;
 }
 
 // ------------------------------------------------------------------ potential terms
 // f(t) = A0 + A env(t) sin(omega t + phi)
-__device__ inline double term_coef(const wp_pot_term& tm, double t) {
+__device__ inline double term_sine(const wp_pot_term& tm, double t) { return sin(tm.omega * t + tm.phi); }
+__device__ inline double term_envelope(const wp_pot_term& tm, double t) {
   double env = 1.0;
   if (tm.env == WP_ENV_GAUSS) {
     const double u = (t - tm.t0) / tm.tau;
@@ -503,7 +520,10 @@ __device__ inline double term_coef(const wp_pot_term& tm, double t) {
       env = 0.0;
     }
   }
-  return tm.A0 + tm.A * env * sin(tm.omega * t + tm.phi);
+  return env;
+}
+__device__ inline double term_coef(const wp_pot_term& tm, double t) {
+  return tm.A0 + tm.A * term_envelope(tm, t) * term_sine(tm, t);
 }
 
 // Additive (non-Gaussian) shape restricted to axis d: the potential is the sum of
@@ -1300,21 +1320,6 @@ __global__ void __launch_bounds__(256, 3) k_pass_batch_f64(const PassParams<doub
   pass_batch_body<double, CONTIG, LOGN>(params, tile_start, block_inst, block_off + blockIdx.x, flags, khalf, raw);
 }
 
-template <class T>
-__device__ void lines_body(const LinesParams<T>& p, int64_t first, int64_t stride);
-
-// Batched per-line records: blockIdx.y selects the instance, x strides over its lines.
-template <class T>
-__global__ void __launch_bounds__(256) k_lines_batch(const LinesParams<T>* __restrict__ params) {
-  __shared__ __align__(16) unsigned char raw[sizeof(LinesParams<T>)];
-  const int* src = reinterpret_cast<const int*>(&params[blockIdx.y]);
-  for (int k = threadIdx.x; k < (int)(sizeof(LinesParams<T>) / sizeof(int)); k += blockDim.x)
-    reinterpret_cast<int*>(raw)[k] = src[k];
-  __syncthreads();
-  const LinesParams<T>& p = *reinterpret_cast<const LinesParams<T>*>(raw);
-  lines_body<T>(p, blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
-}
-
 // Fixed-size pass: n = 2^LOGN points per line, 2048-element tiles, 256 threads.
 // GRID: the variant that also applies a static grid potential (contiguous passes only).
 template <class T, int LOGN, bool CONTIG, bool OBS, bool GRID = false>
@@ -1382,69 +1387,91 @@ __global__ void __launch_bounds__(256) k_lines(const LinesParams<T> p) {
 }
 
 // ------------------------------------------------------------------ per-step tables
-// One block. Forms t = t0 + (step + step_add) dt + t_shift, stores the new step index,
-// and fills, for every axis, the additive potential A_d(x, t), its phase factor
-// exp(-i A_d tau/hbar) (argument reduced by the FP64 sincos), and the Gaussian-term
-// factors; the Gaussian coefficients f_g(t) and f_g(t) tau/hbar go to the control block.
+// Forms t = t0 + (step + step_add) dt + t_shift, stores the new step index, and fills, for
+// every axis, the additive potential A_d(x, t), its phase factor exp(-i A_d tau/hbar), and the
+// Gaussian-term factors; the Gaussian coefficients f_g(t) and f_g(t) tau/hbar go to the
+// control block. With `lines` (2-D) also the line records of the potential pass, whose lines
+// are the entries of axis 0.
+//
+// The kernel is a chain of FP64 latencies (64 clocks an instruction for one warp), so it is
+// laid out for a short chain: the sine and the envelope of a coefficient are formed by
+// different warps, an axis's phases and its Gaussian factors by different threads, and
+// nothing is divided that the host can divide. With the coefficients one after the other,
+// the Gaussian exponentials behind the phases, and the publishing block evaluating the
+// coefficients again, it took 11 us per step (trap and laser) to 14 us (with a Gaussian term).
 template <class T>
 __device__ void prep_body(const PrepParams<T>& p, int blk, int nblk) {
   __shared__ int64_t s_step;
+  __shared__ double fsin[WP_MAX_TERMS], fenv[WP_MAX_TERMS];
   if (threadIdx.x == 0) s_step = p.ctrl->step + p.step_add;
   __syncthreads();
   const int64_t step = s_step;
   const double t = p.g.t0 + (double)step * p.g.dt + p.t_shift;
   const DevPot& pot = *p.pot;
-  __shared__ double fco[WP_MAX_TERMS];
-  if (threadIdx.x < pot.nterms) fco[threadIdx.x] = term_coef(pot.term[threadIdx.x], t);
+  // a block has at least two warps
+  if (threadIdx.x < pot.nterms) fsin[threadIdx.x] = term_sine(pot.term[threadIdx.x], t);
+  if (threadIdx.x >= 32 && threadIdx.x < 32 + pot.nterms) fenv[threadIdx.x - 32] = term_envelope(pot.term[threadIdx.x - 32], t);
   __syncthreads();
-  [[maybe_unused]] const double tau_hbar = p.tau / p.g.hbar;
-  // one flat range over the entries of all axes, so that short axes share a round
+  auto coef = [&](int k) { return pot.term[k].A0 + pot.term[k].A * fenv[k] * fsin[k]; };
+  const double tau_hbar = p.tau_dt * p.dt_hbar;
   const int64_t n01 = p.n[0] + (p.g.ndim > 1 ? p.n[1] : 0);
   const int64_t nall = n01 + (p.g.ndim > 2 ? p.n[2] : 0);
-  for (int64_t e = blk * (int64_t)blockDim.x + threadIdx.x; e < nall; e += (int64_t)nblk * blockDim.x) {
-    {
-      const int d = e < p.n[0] ? 0 : (e < n01 ? 1 : 2);
-      const int64_t i = e - (d == 0 ? 0 : (d == 1 ? p.n[0] : n01));
-      const AxisTab<T>& tb = p.tab[d];
-      const double x = p.g.xmin[d] + (double)i * p.g.dx[d];
-      double A = 0.0;
-      for (int k = 0; k < pot.nterms; k++) {
-        const wp_pot_term& tm = pot.term[k];
-        if (tm.shape == WP_SHAPE_GAUSS) continue;
-        const double part = term_axis_part(tm, d, x, t);
-        if (part != 0.0) A += fco[k] * part;
-      }
-      tb.A[i] = A;
-      if (tb.AT) tb.AT[i] = (T)A;
-      if constexpr (std::is_same<T, float>::value) {
-        // complex64: the factor's high and low parts straight from the float-float cos and
-        // sin of the argument (FP64 only reduces it)
-        ff c, sn;
-        cis_ff(-A * tau_hbar, c, sn);
+  // one flat range over the phases of all axes, then the factors of each Gaussian term
+  for (int64_t w = blk * (int64_t)blockDim.x + threadIdx.x; w < nall * (1 + pot.ngauss);
+       w += (int64_t)nblk * blockDim.x) {
+    const int job = w < nall ? 0 : (w < 2 * nall ? 1 : 2);
+    const int64_t e = w - job * nall;
+    const int d = e < p.n[0] ? 0 : (e < n01 ? 1 : 2);
+    const int64_t i = e - (d == 0 ? 0 : (d == 1 ? p.n[0] : n01));
+    const AxisTab<T>& tb = p.tab[d];
+    const double x = p.g.xmin[d] + (double)i * p.g.dx[d];
+    const bool line = p.lines != nullptr && d == 0;
+    if (job > 0) {
+      const int gg = job - 1, k = pot.gauss_term[gg];
+      const double gf = gauss_axis_factor(pot.term[k], d, x, t);
+      tb.Gd[gg][i] = gf;
+      tb.G[gg][i] = (T)gf;
+      if (line) p.lines[i].g[gg] = (T)(coef(k) * tau_hbar * gf);
+      continue;
+    }
+    double A = 0.0;
+    for (int k = 0; k < pot.nterms; k++) {
+      const wp_pot_term& tm = pot.term[k];
+      if (tm.shape == WP_SHAPE_GAUSS) continue;
+      const double part = term_axis_part(tm, d, x, t);
+      if (part != 0.0) A += coef(k) * part;
+    }
+    tb.A[i] = A;
+    if (tb.AT) tb.AT[i] = (T)A;
+    [[maybe_unused]] TwE<T> lr;
+    if constexpr (std::is_same<T, float>::value) {
+      // complex64: the factor's high and low parts straight from the float-float cos and
+      // sin of the argument (FP64 only reduces it)
+      ff c, sn;
+      cis_ff(-A * tau_hbar, c, sn);
+      tb.P[i] = mk(c.hi, sn.hi);
+      tb.P_lo[i] = mk(c.lo, sn.lo);
+      // on the axis grid, multiples of 2^-11 and the rest, and the line grid, 2^-12
+      auto grid = [&](float M) {
         TwE<float> r;
-        r.h = mk(c.hi, sn.hi);
-        r.l = mk(c.lo, sn.lo);
-        tb.P[i] = r.h;
-        tb.P_lo[i] = r.l;
-        // the same on the axis grid: multiples of 2^-11 and the rest
-        const float M = 6144.0f;
         r.h = mk(__fsub_rn(__fadd_rn(c.hi, M), M), __fsub_rn(__fadd_rn(sn.hi, M), M));
         r.l = mk(__fadd_rn(__fsub_rn(c.hi, r.h.re), c.lo), __fadd_rn(__fsub_rn(sn.hi, r.h.im), sn.lo));
-        tb.Prec[i] = r;
-      } else {
-        double sn, cs;
-        sincos(-A * p.tau / p.g.hbar, &sn, &cs);
-        const T hc = (T)cs, hs = (T)sn;
-        tb.P[i] = mk(hc, hs);
-        tb.P_lo[i] = mk((T)(cs - (double)hc), (T)(sn - (double)hs));
-        tb.Prec[i] = make_rec<T>(cs, sn);
-        if constexpr (std::is_same<T, double>::value) tb.Pfx[i] = fx_rec_of(cs, sn);
-      }
-      for (int gg = 0; gg < pot.ngauss; gg++) {
-        const double gf = gauss_axis_factor(pot.term[pot.gauss_term[gg]], d, x, t);
-        tb.Gd[gg][i] = gf;
-        tb.G[gg][i] = (T)gf;
-      }
+        return r;
+      };
+      tb.Prec[i] = grid(6144.0f);
+      lr = grid(3072.0f);
+    } else {
+      double sn, cs;
+      sincos(-A * tau_hbar, &sn, &cs);
+      const T hc = (T)cs, hs = (T)sn;
+      tb.P[i] = mk(hc, hs);
+      tb.P_lo[i] = mk((T)(cs - (double)hc), (T)(sn - (double)hs));
+      tb.Prec[i] = lr = make_rec<T>(cs, sn);
+      if constexpr (std::is_same<T, double>::value) tb.Pfx[i] = fx_rec_of(cs, sn);
+    }
+    if (line) {
+      p.lines[i].L = lr;
+      for (int gg = pot.ngauss; gg < WP_MAX_GAUSS; gg++) p.lines[i].g[gg] = tzero<T>();
     }
   }
   // The last block to finish publishes the Gaussian coefficients, the table time and the
@@ -1462,10 +1489,9 @@ __device__ void prep_body(const PrepParams<T>& p, int blk, int nblk) {
   __syncthreads();
   if (s_last && threadIdx.x == 0) {
     for (int gg = 0; gg < WP_MAX_GAUSS; gg++) {
-      double fc = 0.0;
-      if (gg < pot.ngauss) fc = term_coef(pot.term[pot.gauss_term[gg]], t);
+      const double fc = gg < pot.ngauss ? coef(pot.gauss_term[gg]) : 0.0;
       p.ctrl->gcoef[gg] = fc;
-      p.ctrl->gphase[gg] = fc * p.tau / p.g.hbar;
+      p.ctrl->gphase[gg] = fc * tau_hbar;
     }
     p.ctrl->t_tab = t;
     p.ctrl->step = step;
@@ -1478,7 +1504,7 @@ __global__ void __launch_bounds__(64) k_prep(const PrepParams<T> p) {
   prep_body<T>(p, blockIdx.x, gridDim.x);
 }
 
-// Batched tables: block b updates instance b. The step increment, the time shift and the
+// Batched tables and line records: block b updates instance b. The step increment, the time shift and the
 // phase length (in units of the instance's dt) are the same for all instances.
 template <class T>
 __global__ void __launch_bounds__(256) k_prep_batch(const PrepParams<T>* __restrict__ params, int step_add,
@@ -1492,7 +1518,8 @@ __global__ void __launch_bounds__(256) k_prep_batch(const PrepParams<T>* __restr
   if (threadIdx.x == 0) {
     p.step_add = step_add;
     p.t_shift = shift_dt * p.g.dt;
-    p.tau = tau_dt * p.g.dt;
+    p.tau_dt = tau_dt;
+    if (tau_dt == 0.0) p.lines = nullptr;
   }
   __syncthreads();
   prep_body<T>(p, 0, 1);
@@ -1676,14 +1703,7 @@ __device__ void res1d_body(const Res1dParams<T>& p, const RS& rs, cx<T>* s) {
       acc[Q_K2] += k * k * rho;
     }
     block_sum(acc, qm, red);
-    if (tid == 0) {
-      const int64_t slot = p.ctrl->nobs;
-      if (slot < p.obs_cap) {
-        finish_obs(qp, qm, p.g, n, p.autocorr, t, s0 + m, p.obs_out + slot * 16);
-        if (!isfinite(p.obs_out[slot * 16 + 1])) p.ctrl->err = WP_ENONFINITE;
-      }
-      p.ctrl->nobs = slot + 1;
-    }
+    if (tid < 32) publish_obs(qp, qm, p.g, p.autocorr, t, s0 + m, tid, p.ctrl, p.obs_out, p.obs_cap);
   }
   if (tid == 0) p.ctrl->step = s0 + m;
 }
@@ -1796,60 +1816,47 @@ __global__ void __launch_bounds__(MAXT) k_res1d_batch(const Res1dParams<T>* __re
 
 #ifdef WP_COMMON_KERNELS
 // ------------------------------------------------------------------ reduction kernel
+// Sum of n rows, stride rows apart, into out (shared) by 256 threads: thread t adds quantity
+// t mod 16 of rows t / 16, t / 16 + 16, .. in order, then 16 threads the 16 parts in order.
+// (One row per thread and a shuffle tree for each of the 16 quantities is 80 dependent FP64 adds
+// more, 5000 clocks.)
+__device__ __forceinline__ void sum_rows(const double* a, int64_t n, int64_t stride, double* out,
+                                         double (*part)[NQ]) {
+  const int q = threadIdx.x & 15, g = threadIdx.x >> 4;
+  double v = 0.0;
+  for (int64_t r = g; r < n; r += 16) v += a[r * stride * NQ + q];
+  part[g][q] = v;
+  __syncthreads();
+  if (threadIdx.x < NQ) {
+    double s = part[0][q];
+#pragma unroll
+    for (int k = 1; k < 16; k++) s += part[k][q];
+    out[q] = s;
+  }
+  __syncthreads();
+}
 // First level: block (b, y) sums rows [b R, b R + R) of the position (y = 0) or momentum
 // (y = 1) partials in a fixed order and leaves the sum in row b R, which no other block
 // reads. The sums are then in rows 0, R, 2R, ... (the partials are scratch of one record).
 __global__ void __launch_bounds__(256) k_reduce_rows(double* pos, int64_t npos, double* mom, int64_t nmom,
                                                      int64_t R) {
-  __shared__ double red[32][NQ];
-  __shared__ double tot[NQ];
+  __shared__ double part[16][NQ], tot[NQ];
   double* a = blockIdx.y ? mom : pos;
   const int64_t n = blockIdx.y ? nmom : npos;
   const int64_t r0 = (int64_t)blockIdx.x * R;
   if (r0 >= n) return;  // the whole block leaves
-  const int64_t r1 = r0 + R < n ? r0 + R : n;
-  double acc[NQ];
-#pragma unroll
-  for (int q = 0; q < NQ; q++) acc[q] = 0.0;
-  for (int64_t r = r0 + threadIdx.x; r < r1; r += blockDim.x) {
-    const double2* row = reinterpret_cast<const double2*>(a + r * NQ);
-#pragma unroll
-    for (int q = 0; q < NQ / 2; q++) {
-      const double2 v = row[q];
-      acc[2 * q] += v.x;
-      acc[2 * q + 1] += v.y;
-    }
-  }
-  block_sum(acc, tot, red);  // every thread has read its rows before the first barrier in it
+  sum_rows(a + r0 * NQ, r0 + R < n ? R : n - r0, 1, tot, part);
   if (threadIdx.x < NQ) a[r0 * NQ + threadIdx.x] = tot[threadIdx.x];
 }
 
 // One block: sums the (first-level) partials in a fixed order and writes the observable
 // record.
 __global__ void __launch_bounds__(256) k_reduce(const ReduceParams p) {
-  __shared__ double red[32][NQ];
-  __shared__ double qp[NQ], qm[NQ];
-  double acc[NQ];
-#pragma unroll
-  for (int q = 0; q < NQ; q++) acc[q] = 0.0;
-  for (int64_t r = threadIdx.x; r < p.npos; r += blockDim.x)
-#pragma unroll
-    for (int q = 0; q < NQ; q++) acc[q] += p.pos[r * p.pos_stride * NQ + q];
-  block_sum(acc, qp, red);
-#pragma unroll
-  for (int q = 0; q < NQ; q++) acc[q] = 0.0;
-  for (int64_t r = threadIdx.x; r < p.nmom; r += blockDim.x)
-#pragma unroll
-    for (int q = 0; q < NQ; q++) acc[q] += p.mom[r * p.mom_stride * NQ + q];
-  block_sum(acc, qm, red);
-  if (threadIdx.x == 0) {
-    const int64_t slot = p.ctrl->nobs;
-    if (slot < p.obs_cap) {
-      finish_obs(qp, qm, p.g, p.ntotal, p.autocorr, p.ctrl->t_tab, p.ctrl->step, p.obs_out + slot * 16);
-      if (!isfinite(p.obs_out[slot * 16 + 1])) p.ctrl->err = WP_ENONFINITE;
-    }
-    p.ctrl->nobs = slot + 1;
-  }
+  __shared__ double part[16][NQ], qp[NQ], qm[NQ];
+  sum_rows(p.pos, p.npos, p.pos_stride, qp, part);
+  sum_rows(p.mom, p.nmom, p.mom_stride, qm, part);
+  if (threadIdx.x < 32)
+    publish_obs(qp, qm, p.g, p.autocorr, p.ctrl->t_tab, p.ctrl->step, threadIdx.x, p.ctrl, p.obs_out, p.obs_cap);
 }
 
 __global__ void k_set_step(Ctrl* c, int64_t step) {

@@ -82,10 +82,11 @@ int launch_pass(const PassParams<T>& p, int64_t ntiles, size_t smem, void* strea
 }
 
 template <class T>
-int launch_prep(const PrepParams<T>& p, void* stream) {
+int launch_prep(const PrepParams<T>& p, int ngauss, void* stream) {
   // 64-thread blocks over the entries of all axes: the FP64 work spreads over SMs
   int64_t nall = 0;
   for (int d = 0; d < p.g.ndim; d++) nall += p.n[d];
+  nall *= 1 + ngauss;
   int64_t blocks = (nall + 63) / 64;
   if (blocks < 1) blocks = 1;
   if (blocks > 512) blocks = 512;
@@ -181,14 +182,6 @@ int launch_pass_batch(const PassParams<T>* params, const int64_t* tile_start, co
 }
 
 template <class T>
-int launch_lines_batch(const LinesParams<T>* params, int ninst, int64_t max_lines, void* stream) {
-  int64_t bx = (max_lines + 255) / 256;
-  if (bx > 64) bx = 64;
-  if (ninst > 0 && bx > 0) k_lines_batch<T><<<dim3((unsigned)bx, (unsigned)ninst), 256, 0, (cudaStream_t)stream>>>(params);
-  return cuda_status(cudaGetLastError());
-}
-
-template <class T>
 int launch_prep_batch(const PrepParams<T>* params, int ninst, int step_add, double shift_dt, double tau_dt,
                       void* stream) {
   if (ninst > 0)
@@ -225,7 +218,7 @@ int launch_res1d_batch(const Res1dParams<T>* params, int ninst, int nthreads, in
   template int pass_smem_limit_set<T>(size_t);                                    \
   template int res1d_smem_limit_set<T>(size_t);                                   \
   template int launch_pass<T>(const PassParams<T>&, int64_t, size_t, void*);     \
-  template int launch_prep<T>(const PrepParams<T>&, void*);                       \
+  template int launch_prep<T>(const PrepParams<T>&, int, void*);                  \
   template int launch_res1d<T>(const Res1dParams<T>&, size_t, void*);            \
   template int launch_convert<T>(const ConvParams<T>&, void*);                    \
   template int launch_static_phase<T>(const StaticPhaseParams<T>&, void*);        \
@@ -236,7 +229,6 @@ int launch_res1d_batch(const Res1dParams<T>* params, int ninst, int nthreads, in
   template int launch_pass_batch<T>(const PassParams<T>*, const int64_t*, const int*, int, int64_t, int64_t, uint32_t, \
                                     int, size_t, void*);                         \
   template int launch_prep_batch<T>(const PrepParams<T>*, int, int, double, double, void*);                    \
-  template int launch_lines_batch<T>(const LinesParams<T>*, int, int64_t, void*);                              \
   template int launch_res1d_batch<T>(const Res1dParams<T>*, int, int, int, int64_t, size_t, void*);
 
 }  // namespace wp

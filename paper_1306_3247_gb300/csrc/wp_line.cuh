@@ -368,22 +368,26 @@ __device__ __forceinline__ void tables(const Res1dParams<T>& p, double t, double
 
 // FP64 sums of the line in a fixed order into `out` (shared memory of block 0): the block's
 // warps in order, then (part: [R][NQ] in block 0, n: which of its two record mbarriers) the
-// blocks.
+// blocks. used: the quantities to sum (a shuffle tree is five dependent FP64 adds, 320 clocks,
+// for each).
 template <class LN>
-__device__ __forceinline__ void total(LN& ln, double (&acc)[NQ], double (*redd)[NQ], double (*part)[NQ], int n,
-                                      double* out) {
+__device__ __forceinline__ void total(LN& ln, double (&acc)[NQ], uint32_t used, double (*redd)[NQ], double (*part)[NQ],
+                                      int n, double* out) {
   const int t = ln.t;
 #pragma unroll
   for (int q = 0; q < NQ; q++) {
-    double v = acc[q];
+    double v = 0.0;
+    if ((used >> q) & 1u) {
+      v = acc[q];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    }
     if ((t & 31) == 0) redd[t >> 5][q] = v;
   }
   ln.bar();
   if (t < NQ) {
-    double v = 0.0;
-    for (int w = 0; w < LN::SH::NW; w++) v += redd[w][t];
+    double v = redd[0][t];
+    for (int w = 1; w < LN::SH::NW; w++) v += redd[w][t];
     if constexpr (LN::R == 1)
       out[t] = v;
     else
@@ -397,8 +401,8 @@ __device__ __forceinline__ void total(LN& ln, double (&acc)[NQ], double (*redd)[
       ln.wait(ln.mb + 4 + n, 0u);
       __syncwarp();
       if (t < NQ) {
-        double v = 0.0;
-        for (int b = 0; b < LN::R; b++) v += part[b][t];
+        double v = part[0][t];
+        for (int b = 1; b < LN::R; b++) v += part[b][t];
         out[t] = v;
       }
     }
@@ -680,7 +684,8 @@ __device__ __forceinline__ void body(const Res1dParams<T>& p, unsigned char* sme
         x[P - 1] = first;
       }
     }
-    total(ln, acc, redd, part[0], 0, qp);
+    const uint32_t ac = p.autocorr ? 3u << Q_AC_RE : 0u;
+    total(ln, acc, ac | (1u << Q_RHO) | (1u << Q_X) | (1u << Q_XX) | (1u << Q_V), redd, part[0], 0, qp);
     ln.template fft<false>(x, tw);
 #pragma unroll
     for (int q = 0; q < NQ; q++) acc[q] = 0.0;
@@ -693,22 +698,20 @@ __device__ __forceinline__ void body(const Res1dParams<T>& p, unsigned char* sme
       acc[Q_K] += kr;
       acc[Q_K2] += kk * kr;
     }
-    total(ln, acc, redd, part[1], 1, qm);
-    if (t == 0 && c == 0u) {
-      for (int e = 0; e < pot.nterms; e++) {
-        if (!((p.plane_mask >> e) & 1u)) continue;
-        const wp_pot_term& tm = pot.term[e];
-        if (tm.shape == WP_SHAPE_LINEAR)
-          qp[Q_V] += fco[0][e] * tm.a[0] * (qp[Q_X] - (tm.c0[0] + tm.v[0] * tm0) * qp[Q_RHO]);
-        else
-          qp[Q_V] += fco[0][e] * qp[Q_RHO];
+    total(ln, acc, (1u << Q_RHOK) | (1u << Q_K) | (1u << Q_K2), redd, part[1], 1, qm);
+    if (t < 32 && c == 0u) {
+      if (t == 0) {
+        for (int e = 0; e < pot.nterms; e++) {
+          if (!((p.plane_mask >> e) & 1u)) continue;
+          const wp_pot_term& tm = pot.term[e];
+          if (tm.shape == WP_SHAPE_LINEAR)
+            qp[Q_V] += fco[0][e] * tm.a[0] * (qp[Q_X] - (tm.c0[0] + tm.v[0] * tm0) * qp[Q_RHO]);
+          else
+            qp[Q_V] += fco[0][e] * qp[Q_RHO];
+        }
       }
-      const int64_t slot = p.ctrl->nobs;
-      if (slot < p.obs_cap) {
-        finish_obs(qp, qm, p.g, N, p.autocorr, tm0, s0 + m, p.obs_out + slot * 16);
-        if (!isfinite(p.obs_out[slot * 16 + 1])) p.ctrl->err = WP_ENONFINITE;
-      }
-      p.ctrl->nobs = slot + 1;
+      __syncwarp();
+      publish_obs(qp, qm, p.g, p.autocorr, tm0, s0 + m, t, p.ctrl, p.obs_out, p.obs_cap);
     }
   }
   if (t == 0 && c == 0u) p.ctrl->step = s0 + m;
