@@ -325,6 +325,11 @@ auto dispatch(const wp_handle* h, F&& f) {
     return expr;                        \
   })
 
+// Axes whose kernels read the stage twiddles with r outermost (AxisTab::Wln).
+bool line_twiddles(const wp_handle* h, int d) {
+  return h->ndim == 1 || (h->prec != WP_C128 && (h->n[d] == 512 || h->n[d] == 1024));
+}
+
 template <class T>
 wp_status alloc_tables(wp_handle* h) {
   // per axis: W, Kfull, Khalf, P (complex T); G[g] (T); A, Gd[g] (double)
@@ -342,7 +347,7 @@ wp_status alloc_tables(wp_handle* h) {
   size_t off_w256[3] = {0, 0, 0};
   size_t off_w2s[3] = {0, 0, 0};
   size_t off_fx[3][4] = {};
-  size_t off_ln = 0;
+  size_t off_ln[3] = {0, 0, 0};
   for (int d = 0; d < h->ndim; d++) {
     const size_t n = (size_t)h->n[d];
     for (int k = 0; k < 4; k++) off[d][k] = add(n * sizeof(cx<T>));
@@ -362,7 +367,7 @@ wp_status alloc_tables(wp_handle* h) {
     off_w2s[d] = (std::is_same<T, float>::value && (n == 64 || n == 128)) ? add(256 * 16) : 0;
     if (std::is_same<T, double>::value)
       for (int k = 0; k < 4; k++) off_fx[d][k] = add(n * sizeof(FxRec));
-    if (h->ndim == 1) off_ln = add(n * (std::is_same<T, double>::value ? sizeof(FxRec) : 16));
+    if (line_twiddles(h, d)) off_ln[d] = add(n * (std::is_same<T, double>::value ? sizeof(FxRec) : 16));
   }
   WP_CUDA(h, dev_malloc(h, &h->tabmem, bytes));
   WP_CUDA(h, cudaMemsetAsync(h->tabmem, 0, bytes, h->stream));
@@ -397,7 +402,7 @@ wp_status alloc_tables(wp_handle* h) {
       tb[d].Kfx_half = (FxRec*)(base + off_fx[d][2]);
       tb[d].Pfx = (FxRec*)(base + off_fx[d][3]);
     }
-    tb[d].Wln = h->ndim == 1 ? (void*)(base + off_ln) : nullptr;
+    tb[d].Wln = line_twiddles(h, d) ? (void*)(base + off_ln[d]) : nullptr;
   }
   // static tables (high and low parts)
   for (int d = 0; d < h->ndim; d++) {
@@ -607,6 +612,7 @@ PassParams<T> pass_params(wp_handle* h, int axis, uint32_t flags, void* in, void
   p.Pfx = tb[axis].Pfx;
   p.Kfx = khalf ? tb[axis].Kfx_half : tb[axis].Kfx_full;
   p.Kfx_half = tb[axis].Kfx_half;
+  p.Wln = tb[axis].Wln;
   p.fx_state = fx_state(h) ? 1 : 0;
   return p;
 }

@@ -206,8 +206,8 @@ struct AxisTab {
   FxRec* Kfx_full;
   FxRec* Kfx_half;
   FxRec* Pfx;
-  // 1-D lines: the stage twiddles with r outermost (twiddle r of index jm at (r - 1) Ns + jm
-  // of its stage), which neighbouring threads read side by side
+  // 1-D lines, and axes of 512 and 1024 points: the stage twiddles with r outermost (twiddle r
+  // of index jm at (r - 1) Ns + jm of its stage), which neighbouring threads read side by side
   void* Wln;
 };
 
@@ -263,6 +263,7 @@ struct PassParams {
   const FxRec* Pfx;
   const FxRec* Kfx;
   const FxRec* Kfx_half;
+  const void* Wln;         // stage twiddles with r outermost (AxisTab), or NULL
   int32_t fx_state;        // every pass of a step runs in fixed point: F_IN_FX, F_OUT_FX apply
 };
 
@@ -458,6 +459,10 @@ int launch_merged_strided(const PassParams<T>* params, const int64_t* tile_start
 template <class T> bool pass256_applies(const PassParams<T>& p);
 template <class T> int launch_pass256(const PassParams<T>& p, void* stream);
 template <class T> int64_t pass256_blocks(const PassParams<T>& p);  // blocks (partial rows) of a launch
+// passes over 512- and 1024-point lines held in registers, complex64 and float-float
+// (wp_linepass_*.cu)
+template <class T> bool line_pass_applies(const PassParams<T>& p);
+template <class T> int launch_line_pass(const PassParams<T>& p, void* stream);
 // complex64 two-stage kernels for 64- and 128-point lines (wp_pass2s_f32.cu), single and
 // batched (class keys kBatchClassP2S + 100 (logn - 6) + v, v as for the 256-point class)
 constexpr int kBatchClassP2S = 1100;

@@ -46,6 +46,7 @@ int launch_pass(const PassParams<T>& p, int64_t ntiles, size_t smem, void* strea
   cudaStream_t st = (cudaStream_t)stream;
   if constexpr (!std::is_same<T, double>::value) {
     if (pass256_applies<T>(p)) return launch_pass256<T>(p, stream);
+    if (line_pass_applies<T>(p)) return launch_line_pass<T>(p, stream);
   }
   if constexpr (std::is_same<T, float>::value) {
     if (pass2s_applies(p)) return launch_pass2s(p, stream);

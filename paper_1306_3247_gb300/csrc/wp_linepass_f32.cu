@@ -1,0 +1,6 @@
+// Passes over 512- and 1024-point lines held in registers for the complex64 form.
+#include <mutex>
+
+#include "wp_linepass.cuh"
+
+WP_LINEPASS_TU(float)
