@@ -327,7 +327,7 @@ auto dispatch(const wp_handle* h, F&& f) {
 
 // Axes whose kernels read the stage twiddles with r outermost (AxisTab::Wln).
 bool line_twiddles(const wp_handle* h, int d) {
-  return h->ndim == 1 || (h->prec != WP_C128 && (h->n[d] == 512 || h->n[d] == 1024));
+  return h->ndim == 1 || (h->prec != WP_C128 && h->n[d] >= 512 && h->n[d] <= 2048);
 }
 
 template <class T>
@@ -1222,7 +1222,7 @@ struct BatchClass1D {
 };
 
 // Blocks off .. off + n - 1 of a pass's class-sorted block list: the instances whose pass
-// axis has 2^logn points (logn 6..10: fixed-size kernel; 0: run-time shape).
+// axis has 2^logn points (logn 5..11: fixed-size kernel; 0: run-time shape).
 struct BatchPassClass {
   int logn = 0;
   int64_t off = 0, n = 0;

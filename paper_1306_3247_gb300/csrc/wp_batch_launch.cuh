@@ -33,12 +33,14 @@ int launch_cls(const PassParams<T>* params, const int64_t* tile_start, const int
   return e == cudaSuccess ? 0 : (int)e;
 }
 
-// One launch for the class of line length 2^logn (6..10: fixed-size kernels; other: run-time shape).
+// One launch for the class of line length 2^logn (5..11: fixed-size kernels; other: run-time shape).
 template <class T, bool CONTIG>
 int launch(const PassParams<T>* params, const int64_t* tile_start, const int* block_inst, int logn,
            int64_t block_off, int64_t nblocks, uint32_t flags, int khalf, size_t smem, void* stream) {
   cudaStream_t st = (cudaStream_t)stream;
   switch (logn) {
+    case 5:
+      return launch_cls<T, CONTIG, 5>(params, tile_start, block_inst, block_off, nblocks, flags, khalf, smem, st);
     case 6:
       return launch_cls<T, CONTIG, 6>(params, tile_start, block_inst, block_off, nblocks, flags, khalf, smem, st);
     case 7:
@@ -49,6 +51,8 @@ int launch(const PassParams<T>* params, const int64_t* tile_start, const int* bl
       return launch_cls<T, CONTIG, 9>(params, tile_start, block_inst, block_off, nblocks, flags, khalf, smem, st);
     case 10:
       return launch_cls<T, CONTIG, 10>(params, tile_start, block_inst, block_off, nblocks, flags, khalf, smem, st);
+    case 11:
+      return launch_cls<T, CONTIG, 11>(params, tile_start, block_inst, block_off, nblocks, flags, khalf, smem, st);
     default:
       return launch_cls<T, CONTIG, 0>(params, tile_start, block_inst, block_off, nblocks, flags, khalf, smem, st);
   }

@@ -1,5 +1,5 @@
-// Host launchers of the fixed-size pass kernels (n = 64..1024 points per line,
-// 2048-element tiles, 256 threads), shared by the per-precision translation units
+// Host launchers of the fixed-size pass kernels (n = 32..2048 points per line, with sums or a
+// grid potential 64..1024; 2048-element tiles, 256 threads), shared by the per-precision translation units
 // wp_fixed_*.cu. OBS selects the variant that also forms the observable partial sums,
 // GRID the one that applies a static grid potential (contiguous passes only).
 #pragma once
@@ -43,40 +43,24 @@ cudaError_t set_limit(int smem) {
   return e;
 }
 
-template <class T, bool OBS, bool GRID>
+template <class T, bool OBS, bool GRID, int LOGN = OBS || GRID ? kFixedObsLogMin : kFixedLogMin>
 int launch(const PassParams<T>& p, unsigned ntiles, size_t smem, void* stream) {
-  cudaStream_t st = (cudaStream_t)stream;
-  cudaError_t e;
-  switch (p.logn) {
-    case 6:
-      e = launch_n<T, OBS, GRID, 6>(p, ntiles, smem, st);
-      break;
-    case 7:
-      e = launch_n<T, OBS, GRID, 7>(p, ntiles, smem, st);
-      break;
-    case 8:
-      e = launch_n<T, OBS, GRID, 8>(p, ntiles, smem, st);
-      break;
-    case 9:
-      e = launch_n<T, OBS, GRID, 9>(p, ntiles, smem, st);
-      break;
-    case 10:
-      e = launch_n<T, OBS, GRID, 10>(p, ntiles, smem, st);
-      break;
-    default:
-      return (int)cudaErrorInvalidConfiguration;
+  if constexpr (LOGN > (OBS || GRID ? kFixedObsLogMax : kFixedLogMax)) {
+    return (int)cudaErrorInvalidConfiguration;
+  } else {
+    if (p.logn != LOGN) return launch<T, OBS, GRID, LOGN + 1>(p, ntiles, smem, stream);
+    return (int)launch_n<T, OBS, GRID, LOGN>(p, ntiles, smem, (cudaStream_t)stream);
   }
-  return e == cudaSuccess ? 0 : (int)e;
 }
 
-template <class T, bool OBS, bool GRID>
+template <class T, bool OBS, bool GRID, int LOGN = OBS || GRID ? kFixedObsLogMin : kFixedLogMin>
 int limit(size_t smem) {
-  cudaError_t e = set_limit<T, OBS, GRID, 6>((int)smem);
-  if (e == cudaSuccess) e = set_limit<T, OBS, GRID, 7>((int)smem);
-  if (e == cudaSuccess) e = set_limit<T, OBS, GRID, 8>((int)smem);
-  if (e == cudaSuccess) e = set_limit<T, OBS, GRID, 9>((int)smem);
-  if (e == cudaSuccess) e = set_limit<T, OBS, GRID, 10>((int)smem);
-  return e == cudaSuccess ? 0 : (int)e;
+  if constexpr (LOGN > (OBS || GRID ? kFixedObsLogMax : kFixedLogMax)) {
+    return 0;
+  } else {
+    const cudaError_t e = set_limit<T, OBS, GRID, LOGN>((int)smem);
+    return e == cudaSuccess ? limit<T, OBS, GRID, LOGN + 1>(smem) : (int)e;
+  }
 }
 
 }  // namespace fixed_detail

@@ -1,7 +1,7 @@
 // Passes of the complex128 form in 64-bit fixed point (wp_fx.h): a tile is held as integers
 // with one exponent through the transforms and factors of the pass. Tiles, stage plan and
 // thread mapping are those of the fixed-shape kernels of wp_kernels.cuh (2048 points, 256
-// threads, n = 64..1024, the lengths whose stages unroll); the passes that form observable
+// threads, n = 32..2048, the lengths whose stages unroll); the passes that form observable
 // sums or apply a grid potential stay in FP64.
 //
 // Bound by the integer pipe (64 lanes per clock; ncu on 256^3: 61 % busy over the launch,
@@ -40,16 +40,17 @@ __device__ __forceinline__ uint32_t tile_sum(uint32_t L, uint32_t& any, uint32_t
 #pragma unroll
   for (int o = C; o < 32; o <<= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
   any = __reduce_or_sync(0xffffffffu, any);
-  if (lane < C) red[warp * C + lane] = L;
+  constexpr int CW = C < 32 ? C : 32;  // lines a warp meets; of 64 lines odd and even warps meet one half each
+  if (lane < CW) red[warp * CW + lane] = L;
   if (lane == 0) redm[warp] = any;
   __syncthreads();
-  uint32_t t = 0;
+  uint32_t t[2] = {0, 0};
 #pragma unroll
   for (int w = 0; w < 8; w++) {
-    t += red[w * C + (lane & (C - 1))];
+    t[C > 32 ? w & 1 : 0] += red[w * CW + (lane & (CW - 1))];
     any |= redm[w];
   }
-  return __reduce_max_sync(0xffffffffu, t);
+  return __reduce_max_sync(0xffffffffu, max(t[0], t[1]));
 }
 // v shifted right by k (the last bit set, as fx_from_double), left for k < 0.
 __device__ __forceinline__ int64_t shift_jam(int64_t v, int32_t k) {

@@ -60,7 +60,10 @@ __host__ __device__ constexpr int wp_stage_tw_offset(int logn, int logNs) {
   }
   return off;
 }
-constexpr int kFixedLogMin = 6, kFixedLogMax = 10;  // fixed-size pass kernels: n = 64..1024
+// Fixed-size pass kernels: n = 32..2048; those that also form observable sums or apply a grid
+// potential, n = 64..1024.
+constexpr int kFixedLogMin = 5, kFixedLogMax = 11;
+constexpr int kFixedObsLogMin = 6, kFixedObsLogMax = 10;
 constexpr int kRes1dLogMin = 8, kRes1dLogMax = 14;  // fixed-length resident lines: n = 256..16384
 
 // A table factor as one 16-byte record: the value for FP64 and float-float, the high
@@ -206,7 +209,7 @@ struct AxisTab {
   FxRec* Kfx_full;
   FxRec* Kfx_half;
   FxRec* Pfx;
-  // 1-D lines, and axes of 512 and 1024 points: the stage twiddles with r outermost (twiddle r
+  // 1-D lines, and axes of 512 to 2048 points: the stage twiddles with r outermost (twiddle r
   // of index jm at (r - 1) Ns + jm of its stage), which neighbouring threads read side by side
   void* Wln;
 };
@@ -432,7 +435,7 @@ template <class T> int pass_smem_limit_set(size_t smem);
 template <class T> int launch_fixed(const PassParams<T>& p, unsigned ntiles, size_t smem, void* stream);
 // One launch per batched pass (wp_batch_merged.cuh): class c of the pass covers launch
 // blocks start[c] .. start[c + 1] - 1 and block-list entries list_off[c] on; key[c] is its
-// line-length class (6..10 fixed-shape, kBatchClassP256 + v two-stage), counted after nprep
+// line-length class (5..11 fixed-shape, kBatchClassP256 + v two-stage), counted after nprep
 // leading blocks that form the per-instance tables (and, for a phase length other than 0, the
 // line records) of the next step, with the step increment, time shift and phase length (units
 // of dt) given.
@@ -459,7 +462,7 @@ int launch_merged_strided(const PassParams<T>* params, const int64_t* tile_start
 template <class T> bool pass256_applies(const PassParams<T>& p);
 template <class T> int launch_pass256(const PassParams<T>& p, void* stream);
 template <class T> int64_t pass256_blocks(const PassParams<T>& p);  // blocks (partial rows) of a launch
-// passes over 512- and 1024-point lines held in registers, complex64 and float-float
+// passes over lines of 512 to 2048 points held in registers, complex64 and float-float
 // (wp_linepass_*.cu)
 template <class T> bool line_pass_applies(const PassParams<T>& p);
 template <class T> int launch_line_pass(const PassParams<T>& p, void* stream);

@@ -746,7 +746,7 @@ __device__ void line_factors(const PassParams<T>& p, const cx<T>* const* H, cons
 // Shape of a pass: tile lines C = 2^logC, line length n = 2^logn, shared-memory row
 // stride LS, contiguous or strided axis, block size. DynShape holds them at run time;
 // FixShape makes them compile-time constants so that every index folds and the stage
-// sequence unrolls (used for n = 64..1024, the common grid sizes).
+// sequence unrolls (used for n = 32..2048, the common grid sizes).
 struct DynShape {
   static constexpr bool fixed = false;
   int logn, logC, LS, nthr;
@@ -1222,7 +1222,7 @@ __global__ void __launch_bounds__(32 * E) k_pass(const PassParams<T> p) {
 // block_off + b of the class-sorted block list (tile_start[k]: first block of instance k),
 // serving tile (block - tile_start[inst]) of instance block_inst[block]. Every instance
 // tiles its lines into 2048-element tiles with 256 threads. The block copies its
-// instance's parameters to shared memory and runs the pass body: LOGN = 6..10 the
+// instance's parameters to shared memory and runs the pass body: LOGN = 5..11 the
 // compile-time-shape body (with per-line records), LOGN = 0 the run-time one.
 // raw: a 16-byte aligned shared-memory buffer of sizeof(PassParams<T>) bytes for the
 // instance's parameters (the caller's, so that several bodies in one kernel share it).
@@ -1309,7 +1309,7 @@ __global__ void __launch_bounds__(256) k_pass_batch(const PassParams<T>* __restr
   __shared__ __align__(16) unsigned char raw[sizeof(PassParams<T>)];
   pass_batch_body<T, CONTIG, LOGN>(params, tile_start, block_inst, block_off + blockIdx.x, flags, khalf, raw);
 }
-// complex128 with a compile-time shape (LOGN = 6..10): the fixed-point pass, three blocks
+// complex128 with a compile-time shape (LOGN = 5..11): the fixed-point pass, three blocks
 // per SM as alone.
 template <bool CONTIG, int LOGN>
 __global__ void __launch_bounds__(256, 3) k_pass_batch_f64(const PassParams<double>* __restrict__ params,

@@ -1,4 +1,4 @@
-// Passes over lines of 512 and 1024 points held in registers (complex64, float-float): thread t
+// Passes over lines of 512, 1024 and 2048 points held in registers (complex64, float-float): thread t
 // of a line's n/8 threads has the points t + k n/8, which are the points of its butterfly in
 // the first Stockham stage and its outputs in the last one. A tile is therefore read from and
 // written to global memory directly, the factors between two transforms apply in registers,
@@ -27,12 +27,12 @@ template <class T, int LOGN, bool CONTIG, bool WIDE>
 struct Shape {
   static constexpr int N = 1 << LOGN, TL = N / 8;  // threads per line
   // lines per block: 128 threads of a contiguous axis, a sector or two of columns of a strided one
-  static constexpr int C = CONTIG ? 128 / TL : (WIDE ? 64 : 32) / (int)sizeof(cx<T>);
+  static constexpr int C = CONTIG ? (TL < 128 ? 128 / TL : 1) : (WIDE ? 64 : 32) / (int)sizeof(cx<T>);
   static constexpr int LOGC = C == 8 ? 3 : (C == 4 ? 2 : (C == 2 ? 1 : 0));
   static constexpr int NT = TL * C;
   static constexpr int LINE = N + N / 8;
   static constexpr size_t SMEM = (size_t)C * LINE * sizeof(cx<T>);
-  static constexpr int MIN_BLOCKS = (sizeof(cx<T>) == 8 ? 1024 : 512) / NT;
+  static constexpr int MIN_BLOCKS = (sizeof(cx<T>) == 8 ? 1024 : 512) / NT;  // 64 or 128 registers
 };
 
 template <class T, int LOGN, bool CONTIG, bool WIDE>
@@ -152,11 +152,11 @@ __global__ void __launch_bounds__(Shape<T, LOGN, CONTIG, WIDE>::NT, Shape<T, LOG
   for (int k = 0; k < 8; k++) out[k * step] = x[k];
 }
 
-// Passes these kernels serve: 512 or 1024 points under the fixed schedule, no sums, no grid
+// Passes these kernels serve: 512 to 2048 points under the fixed schedule, no sums, no grid
 // potential, whole tiles.
 template <class T>
 bool applies(const PassParams<T>& p) {
-  if (!p.fixed || !p.Wln || (p.logn != 9 && p.logn != 10)) return false;
+  if (!p.fixed || !p.Wln || p.logn < 9 || p.logn > 11) return false;
   const uint32_t f = p.flags;
   if (f & (F_OBS_POS | F_OBS_MOM | F_NO_STORE | F_AUTOCORR)) return false;
   if (p.grid_rec && (f & F_PHASE)) return false;
@@ -192,8 +192,9 @@ cudaError_t launch_n(const PassParams<T>& p, cudaStream_t st) {
     // Two sectors a row once the state is beyond L2's half (64 MB), where DRAM gives single
     // sectors at a lower rate: the float-float kinetic pass of 512^3 takes 3708 us with one
     // sector and 2623 with two. Below, smaller blocks fill the chip better.
-    if (p.log_inner >= 3 && (sizeof(cx<T>) << lntot) > ((size_t)64 << 20))
-      return kin ? go<T, LOGN, false, true, 0, false, true>(p, st) : go<T, LOGN, false, true, 0, false, false>(p, st);
+    if constexpr (LOGN <= 10)
+      if (p.log_inner >= 3 && (sizeof(cx<T>) << lntot) > ((size_t)64 << 20))
+        return kin ? go<T, LOGN, false, true, 0, false, true>(p, st) : go<T, LOGN, false, true, 0, false, false>(p, st);
     return kin ? go<T, LOGN, false, false, 0, false, true>(p, st) : go<T, LOGN, false, false, 0, false, false>(p, st);
   }
   const int ng = p.flags & F_PHASE ? p.ngauss : 0;
@@ -214,7 +215,9 @@ cudaError_t launch_n(const PassParams<T>& p, cudaStream_t st) {
   }                                                                                              \
   template <>                                                                                    \
   int launch_line_pass<T>(const PassParams<T>& p, void* stream) {                                \
-    return (int)(p.logn == 9 ? lp::launch_n<T, 9>(p, (cudaStream_t)stream)                       \
-                             : lp::launch_n<T, 10>(p, (cudaStream_t)stream));                    \
+    cudaStream_t st = (cudaStream_t)stream;                                                      \
+    return (int)(p.logn == 9    ? lp::launch_n<T, 9>(p, st)                                      \
+                 : p.logn == 10 ? lp::launch_n<T, 10>(p, st)                                     \
+                                : lp::launch_n<T, 11>(p, st));                                   \
   }                                                                                              \
   }

@@ -1,4 +1,4 @@
-// Passes over 512- and 1024-point lines held in registers for the complex64 form.
+// Passes over 512- to 2048-point lines held in registers for the complex64 form.
 #include <mutex>
 
 #include "wp_linepass.cuh"

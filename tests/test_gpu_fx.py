@@ -100,3 +100,37 @@ def test_not_finite(shape):
         with pytest.raises(WPK.WavepacketError):
             P.run(4, 4)
         assert np.all(np.isnan(P.get_state()))
+
+
+@pytest.mark.parametrize("prec,tol", [("c128", 1e-13), ("c64", 1e-5), ("c128f", 1e-11)])
+@pytest.mark.parametrize("shape", [(32, 64), (64, 32), (32, 2048), (2048, 64), (2048, 4), (4, 2048), (32, 64, 64),
+                                   (128, 32, 64), (64, 64, 32)])
+def test_axes_of_32_and_2048(shape, prec, tol):
+    """The shortest and longest compile-time lines: transforms, and runs with records (formed
+    by the run-time kernels at these lengths) and without."""
+    nd = len(shape)
+    rng = np.random.default_rng(sum(shape))
+    x = rng.standard_normal(shape) + 1j * rng.standard_normal(shape)
+    pb, terms = problem(shape), TERMS["both"](nd)
+    psi0 = O.gaussian(pb, [0.3, -0.4, 0.2][:nd], [1.0, -0.5, 0.3][:nd], [1.0, 0.8, 0.9][:nd])
+    ref, ref_obs = O.run(pb, terms, psi0, 30, 15)
+    with WPK.Propagator(pb, terms, prec) as P:
+        P.set_state(x)
+        P.fft(-1)
+        assert rel_l2(P.get_state(), np.fft.fftn(x)) < (1e-15 if prec == "c128" else tol)
+        P.set_state(psi0)
+        obs = WPK.obs_matrix(P.run(30, 15))
+        assert rel_l2(P.get_state(), ref) < tol
+        P.set_state(psi0)
+        P.step_index = 0
+        P.step(30)
+        alone = P.get_state()
+        assert rel_l2(alone, ref) < tol
+    scale = np.maximum(np.max(np.abs(ref_obs), axis=0), 1.0)
+    assert np.max(np.abs(obs[:, :14] - ref_obs[:, :14]) / scale[:14]) < 10 * tol
+    if nd == 2:
+        with WPK.Batch(prec) as B:
+            B.add(pb, terms)
+            B.set_state(0, psi0)
+            B.step(30)
+            assert np.array_equal(alone, B.get_state(0))

@@ -1,4 +1,4 @@
-"""Passes over 512- and 1024-point lines held in registers (complex64, float-float): equal to
+"""Passes over lines of 512 to 2048 points held in registers (complex64, float-float): equal to
 the batched kernels of the same instance bit for bit (other tiles, the same stages and factors),
 and to the oracle within the forms' bounds (20 steps: complex64 1e-5, float-float 1e-11
 relative in 2-norm), for every potential kind, both orders and transforms alone, down to
@@ -36,7 +36,9 @@ def cut(terms, nd):
 @pytest.mark.parametrize("order", ["vkv", "kvk"])
 @pytest.mark.parametrize("shape,terms", [((512, 1024), [QUAD, DRIVE]), ((1024, 512), [BUMP]),
                                          ((1024, 64), [QUAD, BUMP]), ((64, 512), [BUMP, WALL]),
-                                         ((512, 512), [QUAD, BUMP, WALL]), ((1024, 4), [QUAD])])
+                                         ((512, 512), [QUAD, BUMP, WALL]), ((1024, 4), [QUAD]),
+                                         ((2048, 64), [QUAD, BUMP, WALL]), ((64, 2048), [BUMP]),
+                                         ((2048, 4), [QUAD, DRIVE]), ((4, 2048), [QUAD])])
 def test_alone_batched_and_oracle(shape, terms, order, prec):
     pb, terms = problem(shape, order), cut(terms, len(shape))
     psi0 = O.gaussian(pb, [0.5, -0.4], [1.0, -0.5], [1.3, 1.1])
@@ -53,7 +55,8 @@ def test_alone_batched_and_oracle(shape, terms, order, prec):
 
 
 @pytest.mark.parametrize("prec", ["c64", "c128f"])
-@pytest.mark.parametrize("shape", [(512, 32, 64), (32, 1024, 16), (16, 64, 512)])
+@pytest.mark.parametrize("shape", [(512, 32, 64), (32, 1024, 16), (16, 64, 512),
+                                   (2048, 8, 16), (8, 2048, 16), (16, 4, 2048)])
 def test_three_axes(shape, prec):
     pb, terms = problem(shape, "vkv"), [QUAD, BUMP]
     psi0 = O.gaussian(pb, [0.5, -0.4, 0.2], [1.0, -0.5, 0.0], [1.3, 1.1, 1.6])
