@@ -242,6 +242,7 @@ PassPlan make_plan(const wp_handle* h, int axis, const wp_schedule& sc) {
   p.max_radix_log = sc.max_radix_log;
   p.fixed = sc.fixed && (p.logn >= kFixedLogMin && p.logn <= kFixedLogMax && p.logC == kTileLog - p.logn &&
                          p.nthreads == 256 && p.ept == 8);
+  if (p.fixed && h->prec == WP_C128) p.smem = kFxTileBytes;
   return p;
 }
 
@@ -327,7 +328,7 @@ auto dispatch(const wp_handle* h, F&& f) {
 
 // Axes whose kernels read the stage twiddles with r outermost (AxisTab::Wln).
 bool line_twiddles(const wp_handle* h, int d) {
-  return h->ndim == 1 || (h->prec != WP_C128 && h->n[d] >= 512 && h->n[d] <= 2048);
+  return h->ndim == 1 || h->prec == WP_C128 || (h->n[d] >= 512 && h->n[d] <= 2048);
 }
 
 template <class T>
@@ -346,7 +347,7 @@ wp_status alloc_tables(wp_handle* h) {
   size_t off_obs[3][3];
   size_t off_w256[3] = {0, 0, 0};
   size_t off_w2s[3] = {0, 0, 0};
-  size_t off_fx[3][4] = {};
+  size_t off_fx[3][3] = {};
   size_t off_ln[3] = {0, 0, 0};
   for (int d = 0; d < h->ndim; d++) {
     const size_t n = (size_t)h->n[d];
@@ -366,7 +367,7 @@ wp_status alloc_tables(wp_handle* h) {
     off_w256[d] = (!std::is_same<T, double>::value && n == 256) ? add(256 * 16) : 0;
     off_w2s[d] = (std::is_same<T, float>::value && (n == 64 || n == 128)) ? add(256 * 16) : 0;
     if (std::is_same<T, double>::value)
-      for (int k = 0; k < 4; k++) off_fx[d][k] = add(n * sizeof(FxRec));
+      for (int k = 0; k < 3; k++) off_fx[d][k] = add(n * sizeof(FxRec));
     if (line_twiddles(h, d)) off_ln[d] = add(n * (std::is_same<T, double>::value ? sizeof(FxRec) : 16));
   }
   WP_CUDA(h, dev_malloc(h, &h->tabmem, bytes));
@@ -397,10 +398,9 @@ wp_status alloc_tables(wp_handle* h) {
     tb[d].W2s = (std::is_same<T, float>::value && (h->n[d] == 64 || h->n[d] == 128)) ? (void*)(base + off_w2s[d])
                                                                                      : nullptr;
     if (std::is_same<T, double>::value) {
-      tb[d].Wfx = (FxRec*)(base + off_fx[d][0]);
-      tb[d].Kfx_full = (FxRec*)(base + off_fx[d][1]);
-      tb[d].Kfx_half = (FxRec*)(base + off_fx[d][2]);
-      tb[d].Pfx = (FxRec*)(base + off_fx[d][3]);
+      tb[d].Kfx_full = (FxRec*)(base + off_fx[d][0]);
+      tb[d].Kfx_half = (FxRec*)(base + off_fx[d][1]);
+      tb[d].Pfx = (FxRec*)(base + off_fx[d][2]);
     }
     tb[d].Wln = line_twiddles(h, d) ? (void*)(base + off_ln[d]) : nullptr;
   }
@@ -436,7 +436,7 @@ wp_status alloc_tables(wp_handle* h) {
       // then (FP32 only) low part
       const int logn = h->g.ln[d];
       std::vector<unsigned char> rec(n * 16, 0);
-      std::vector<FxRec> fx(tb[d].Wfx ? n : 0, FxRec{});
+      std::vector<FxRec> fx(std::is_same<T, double>::value ? n : 0, FxRec{});
       const long double pi = 3.141592653589793238462643383279502884L;
       int ls = 0;
       while (ls < logn) {
@@ -459,7 +459,6 @@ wp_status alloc_tables(wp_handle* h) {
         ls += lr;
       }
       WP_CUDA(h, cudaMemcpy(tb[d].Wst, rec.data(), rec.size(), cudaMemcpyHostToDevice));
-      if (!fx.empty()) WP_CUDA(h, cudaMemcpy(tb[d].Wfx, fx.data(), n * sizeof(FxRec), cudaMemcpyHostToDevice));
       if (tb[d].Wln) {
         const size_t rb = fx.empty() ? 16 : sizeof(FxRec);
         const unsigned char* from = fx.empty() ? rec.data() : (const unsigned char*)fx.data();
@@ -608,7 +607,6 @@ PassParams<T> pass_params(wp_handle* h, int axis, uint32_t flags, void* in, void
   p.grid_rec = (h->vgrid && h->phase_half >= 0) ? (const TwE<T>*)h->vgrid_rec[h->phase_half] : nullptr;
   p.W256 = tb[axis].W256;
   p.W2s = tb[axis].W2s;
-  p.Wfx = tb[axis].Wfx;
   p.Pfx = tb[axis].Pfx;
   p.Kfx = khalf ? tb[axis].Kfx_half : tb[axis].Kfx_full;
   p.Kfx_half = tb[axis].Kfx_half;

@@ -30,28 +30,129 @@ __device__ __forceinline__ uint32_t wlo(double x) { return (uint32_t)__double2lo
 __device__ __forceinline__ uint32_t absh(uint32_t h) { return h ^ (uint32_t)((int32_t)h >> 31); }
 __device__ __forceinline__ uint32_t absh(int64_t v) { return absh((uint32_t)(v >> 32)); }
 
-// The largest line sum of the tile (L: the thread's part of line tid mod C's) and the union
-// of the threads' `any`. red, redm: 256 and 8 words, not used by anything else between the
-// barriers before and after the call.
-template <int LOGC>
-__device__ __forceinline__ uint32_t tile_sum(uint32_t L, uint32_t& any, uint32_t* red, uint32_t* redm) {
-  constexpr int C = 1 << LOGC;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int o = C; o < 32; o <<= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
-  any = __reduce_or_sync(0xffffffffu, any);
-  constexpr int CW = C < 32 ? C : 32;  // lines a warp meets; of 64 lines odd and even warps meet one half each
-  if (lane < CW) red[warp * CW + lane] = L;
-  if (lane == 0) redm[warp] = any;
-  __syncthreads();
-  uint32_t t[2] = {0, 0};
-#pragma unroll
-  for (int w = 0; w < 8; w++) {
-    t[C > 32 ? w & 1 : 0] += red[w * CW + (lane & (CW - 1))];
-    any |= redm[w];
+// A tile's lines in registers and shared memory: thread t of a line's n/8 threads holds the
+// points t + k n/8, which are the inputs of its butterfly in the first Stockham stage and its
+// outputs in the last; shared memory is crossed between the stages of a transform only, and
+// one in eight of its places is left free against bank conflicts. Contiguous axes: a line's
+// threads side by side (whole sectors, and for n <= 256 a line within a warp, which then needs
+// no block barrier between stages); strided axes: the tile's lines, adjacent columns, side by
+// side.
+template <int LOGN, bool CONTIG>
+struct Tile {
+  static constexpr int N = 1 << LOGN, LOGTL = LOGN - 3, TL = 1 << LOGTL, LOGC = 11 - LOGN, C = 1 << LOGC;
+  static constexpr int LINE = N + N / 8;
+  static_assert(C * LINE * sizeof(cx<int64_t>) == kFxTileBytes, "");
+  cx<int64_t>* s;
+  int t, l;
+  __device__ __forceinline__ explicit Tile(void* smem)
+      : s(reinterpret_cast<cx<int64_t>*>(smem)),
+        t(CONTIG ? threadIdx.x & (TL - 1) : threadIdx.x >> LOGC),
+        l(CONTIG ? threadIdx.x >> LOGTL : threadIdx.x & (C - 1)) {}
+  // offset of the thread's point 0, and the distance of the next
+  __device__ __forceinline__ int64_t base(int log_inner, int64_t tile, int64_t& step) const {
+    if (CONTIG) {
+      step = TL;
+      return (((tile << LOGC) + l) << LOGN) + t;
+    }
+    const int tpo = log_inner - LOGC;
+    const int64_t o0 = tile >> tpo, cb = (tile & ((int64_t(1) << tpo) - 1)) << LOGC;
+    step = int64_t(TL) << log_inner;
+    return (((o0 << LOGN) + t) << log_inner) + cb + l;
   }
-  return __reduce_max_sync(0xffffffffu, max(t[0], t[1]));
-}
+  // index of the thread's line in the pass's line records
+  __device__ __forceinline__ int64_t line(int log_inner, int64_t tile) const {
+    if (CONTIG) return (tile << LOGC) + l;
+    return ((tile & ((int64_t(1) << (log_inner - LOGC)) - 1)) << LOGC) + l;
+  }
+  __device__ __forceinline__ cx<int64_t>& at(int i) const {
+    const int q = i + (i >> 3);
+    return CONTIG ? s[l * LINE + q] : s[q * C + l];
+  }
+  __device__ __forceinline__ static void sync() {
+    if constexpr (CONTIG && TL <= 32)
+      __syncwarp();
+    else
+      __syncthreads();
+  }
+
+  // The largest line sum of the tile (L: the thread's part of its line's) and the union of
+  // the threads' `any`. red, redm: 256 and 8 words, not used by anything else between the
+  // barriers before and after the call.
+  __device__ __forceinline__ uint32_t sum(uint32_t L, uint32_t& any, uint32_t* red, uint32_t* redm) const {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    any = __reduce_or_sync(0xffffffffu, any);
+    if (lane == 0) redm[warp] = any;
+    uint32_t r = 0;
+    if constexpr (CONTIG) {
+#pragma unroll
+      for (int o = 1; o < (TL < 32 ? TL : 32); o <<= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
+      if constexpr (TL < 32) L = __reduce_max_sync(0xffffffffu, L);
+      if (lane == 0) red[warp] = L;
+      __syncthreads();
+      constexpr int WL = TL < 32 ? 1 : TL / 32;  // warps of a line
+#pragma unroll
+      for (int w = 0; w < 8; w += WL) {
+        uint32_t u = 0;
+#pragma unroll
+        for (int k = 0; k < WL; k++) u += red[w + k];
+        r = max(r, u);
+      }
+    } else {
+      constexpr int CW = C < 32 ? C : 32;  // lines a warp meets; of 64 lines odd and even warps meet one half each
+#pragma unroll
+      for (int o = C; o < 32; o <<= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
+      if (lane < CW) red[warp * CW + lane] = L;
+      __syncthreads();
+      uint32_t u[2] = {0, 0};
+#pragma unroll
+      for (int w = 0; w < 8; w++) u[C > 32 ? w & 1 : 0] += red[w * CW + (lane & (CW - 1))];
+      r = __reduce_max_sync(0xffffffffu, max(u[0], u[1]));
+    }
+#pragma unroll
+    for (int w = 0; w < 8; w++) any |= redm[w];
+    return r;
+  }
+
+  // The forward transform of the tile's lines, with the scaling of sc. The inverse one is the
+  // same on points with real and imaginary parts exchanged, before and after.
+  template <int LOGNS = 0, int S = 0>
+  __device__ __forceinline__ void fft(cx<int64_t> (&x)[8], const FxRec* __restrict__ tw, const FxSchedule& sc) const {
+    constexpr int LR = wp_stage_radix_log(LOGN, LOGNS), R = 1 << LR, B = 8 / R, NS = 1 << LOGNS;
+    if constexpr (LOGNS > 0) {
+#pragma unroll
+      for (int k = 0; k < 8; k++) x[k] = at(t + k * TL);
+    }
+#pragma unroll
+    for (int b = 0; b < B; b++) {
+      cx<int64_t> v[R];
+#pragma unroll
+      for (int r = 0; r < R; r++) v[r] = x[b + B * r];
+      if constexpr (LOGNS > 0) {
+        const uint32_t sh = sc.at[S];
+        const FxRec* e = tw + wp_stage_tw_offset(LOGN, LOGNS) + ((t + b * TL) & (NS - 1));
+        v[0] = mk(v[0].re >> (2u - sh), v[0].im >> (2u - sh));
+#pragma unroll
+        for (int r = 1; r < R; r++) v[r] = fx_cmul(v[r], e[(r - 1) * NS], sh);
+      }
+      fx_dft<R>(v);
+#pragma unroll
+      for (int r = 0; r < R; r++) x[b + B * r] = v[r];
+    }
+    if constexpr (LOGNS + LR < LOGN) {
+      sync();  // the reads of the stage (or transform) before are done
+#pragma unroll
+      for (int b = 0; b < B; b++) {
+        const int j = t + b * TL;
+        const int d0 = ((j >> LOGNS) << (LOGNS + LR)) + (j & (NS - 1));
+#pragma unroll
+        for (int r = 0; r < R; r++) at(d0 + (r << LOGNS)) = x[b + B * r];
+      }
+      sync();
+      fft<LOGNS + LR, S + 1>(x, tw, sc);
+    }
+  }
+};
+
 // v shifted right by k (the last bit set, as fx_from_double), left for k < 0.
 __device__ __forceinline__ int64_t shift_jam(int64_t v, int32_t k) {
   if (k < 0) return (int64_t)((uint64_t)v << -k);
@@ -59,54 +160,9 @@ __device__ __forceinline__ int64_t shift_jam(int64_t v, int32_t k) {
   return (int64_t)(((uint64_t)(uint32_t)((int32_t)(v >> 32) >> k) << 32) | lo);
 }
 
-// One Stockham stage (stage_fixed) with its scaling.
-template <int LOGN, int LOGC, int LS, int LOGNS>
-__device__ __forceinline__ void stage(cx<int64_t>* s, const FxRec* __restrict__ tw, uint32_t sh, int tid) {
-  constexpr int LR = wp_stage_radix_log(LOGN, LOGNS);
-  constexpr int R = 1 << LR, C = 1 << LOGC, NR = 1 << (LOGN - LR), B = 8 / R, NS = 1 << LOGNS;
-  cx<int64_t> v[B][R];
+__device__ __forceinline__ void exchange(cx<int64_t> (&x)[8]) {
 #pragma unroll
-  for (int b = 0; b < B; b++) {
-    const int bi = tid + b * 256, l = bi & (C - 1), j = bi >> LOGC;
-#pragma unroll
-    for (int r = 0; r < R; r++) v[b][r] = s[(j + r * NR) * LS + l];
-    if (LOGNS > 0) {
-      const FxRec* e = tw + (j & (NS - 1)) * (R - 1);
-      v[b][0] = mk(v[b][0].re >> (2u - sh), v[b][0].im >> (2u - sh));
-#pragma unroll
-      for (int r = 1; r < R; r++) v[b][r] = fx_cmul(v[b][r], e[r - 1], sh);
-    }
-    fx_dft<R>(v[b]);
-  }
-  __syncthreads();
-#pragma unroll
-  for (int b = 0; b < B; b++) {
-    const int bi = tid + b * 256, l = bi & (C - 1), j = bi >> LOGC;
-    const int d0 = ((j >> LOGNS) << (LOGNS + LR)) + (j & (NS - 1));
-#pragma unroll
-    for (int r = 0; r < R; r++) s[(d0 + (r << LOGNS)) * LS + l] = v[b][r];
-  }
-  __syncthreads();
-}
-// The forward transform of every line of the tile. The inverse one is the same on points
-// with real and imaginary parts exchanged, before and after.
-template <int LOGN, int LOGC, int LS, int LOGNS = 0, int T = 0>
-__device__ __forceinline__ void fft(cx<int64_t>* s, const FxRec* __restrict__ tw, const FxSchedule& sc, int tid) {
-  if constexpr (LOGNS < LOGN) {
-    stage<LOGN, LOGC, LS, LOGNS>(s, tw + wp_stage_tw_offset(LOGN, LOGNS), sc.at[T], tid);
-    fft<LOGN, LOGC, LS, LOGNS + wp_stage_radix_log(LOGN, LOGNS), T + 1>(s, tw, sc, tid);
-  }
-}
-
-// Point e of the tile, its parts exchanged when swap is 1.
-__device__ __forceinline__ void put(cx<int64_t>* s, int e, int swap, int64_t re, int64_t im) {
-  int64_t* q = reinterpret_cast<int64_t*>(s + e);
-  q[swap] = re;
-  q[1 - swap] = im;
-}
-__device__ __forceinline__ cx<int64_t> get(const cx<int64_t>* s, int e, int swap) {
-  const int64_t* q = reinterpret_cast<const int64_t*>(s + e);
-  return mk(q[swap], q[1 - swap]);
+  for (int k = 0; k < 8; k++) x[k] = mk(x[k].im, x[k].re);
 }
 
 // The factor exp(-i theta) of a Gaussian term (FP64, as apply_gauss_phase).
@@ -124,24 +180,35 @@ __device__ __noinline__ cx<double> scaled(cx<T> x, int e) {
   return mk(scalbn(__ll2double_rn(x.re), e), scalbn(__ll2double_rn(x.im), e));
 }
 
-// v: the thread's points i0 + k 256/C of line tid mod C (fixed_walk), loaded by the caller.
+// The Gaussian terms of the thread's points in shared memory, one point at a time: the
+// sine's code and registers once, and none of the pass's registers live across it.
+template <class TI>
+__device__ __noinline__ int gauss_points(TI ti, double a0, double a1, const double* G0, const double* G1) {
+  int bad = 0;
+#pragma unroll 1
+  for (int k = 0; k < 8; k++) {
+    const int i = ti.t + k * TI::TL;
+    cx<int64_t> y = ti.at(i);
+    if (gauss_line_active(a0)) y = gauss_phase(y, a0 * G0[i], bad);
+    if (gauss_line_active(a1)) y = gauss_phase(y, a1 * G1[i], bad);
+    ti.at(i) = y;
+  }
+  return bad;
+}
+
+// v: the thread's points, loaded by the caller.
 template <int LOGN, bool CONTIG>
-__device__ __forceinline__ void pass(const PassParams<double>& p, cx<int64_t>* s, int64_t tile, cx<double> (&v)[8]) {
-  using SH = FixShape<LOGN, CONTIG>;
-  constexpr int LOGC = SH::logC, C = 1 << LOGC, LS = SH::LS, ISTEP = 256 >> LOGC;
+__device__ __forceinline__ void pass(const PassParams<double>& p, void* smem, int64_t tile, cx<double> (&v)[8]) {
+  using TI = Tile<LOGN, CONTIG>;
+  constexpr int TL = TI::TL;
   __shared__ uint32_t red[2][256];
   __shared__ uint32_t redm[3][8];
-  __shared__ int spoil;  // a factor that is not finite spoils its tile
-  const int tid = threadIdx.x, l = tid & (C - 1), i0 = tid >> LOGC;
+  const TI ti(smem);
+  const int tid = threadIdx.x;
   const uint32_t f = p.flags;
-  const FxRec* tw = p.Wfx;
-
-  int64_t o0, cb, base, es;
-  int ll, ii;
-  tile_origin(p, SH(), tile, o0, cb);
-  fixed_walk<double, SH>(p, o0, cb, ll, ii, base, es);
-  cx<double>* dst = p.out + base;
-  const int64_t step = es * ISTEP;
+  const FxRec* tw = reinterpret_cast<const FxRec*>(p.Wln);
+  int64_t step;
+  cx<double>* dst = p.out + ti.base(p.log_inner, tile, step);
   const bool in_fx = (f & F_IN_FX) && p.fx_state, out_fx = (f & F_OUT_FX) && p.fx_state;
 
   // Load: the tile's exponent (the largest leading bit), its bounds M and S, the integers.
@@ -149,7 +216,6 @@ __device__ __forceinline__ void pass(const PassParams<double>& p, cx<int64_t>* s
   auto tile_max = [&](uint32_t m) {
     m = __reduce_max_sync(0xffffffffu, m);
     if ((tid & 31) == 0) redm[0][tid >> 5] = m;
-    if (tid == 0) spoil = 0;
     __syncthreads();
 #pragma unroll
     for (int w = 0; w < 8; w++) m = max(m, redm[0][w]);
@@ -164,8 +230,9 @@ __device__ __forceinline__ void pass(const PassParams<double>& p, cx<int64_t>* s
   FxSchedule sc;
   int32_t ex;
   uint32_t L = 0;
-  const bool ph = (f & F_PHASE) != 0, kin = (f & F_KIN) != 0;
-  int swap = (f & F_IFFT) ? 1 : 0;  // whether the tile's points have their parts exchanged
+  const bool ph = CONTIG && (f & F_PHASE), kin = !CONTIG && (f & F_KIN);
+  bool swap = (f & F_IFFT) != 0;  // whether the points have their parts exchanged
+  cx<int64_t> x[8];
   if (in_fx) {
     uint32_t m = 0;
 #pragma unroll
@@ -180,15 +247,15 @@ __device__ __forceinline__ void pass(const PassParams<double>& p, cx<int64_t>* s
       any |= ar | ai;
       L += (ar >> 11) + (ai >> 11) + 2u;
     }
-    const uint32_t Lm = tile_sum<LOGC>(L, any, red[0], redm[1]);
+    const uint32_t Lm = ti.sum(L, any, red[0], redm[1]);
     sc = fx_schedule<LOGN>(65 - __clz((int)any), fx_sum_bits(Lm));
     ex = (int32_t)m - kFxBias + sc.first;
     const uint32_t right = sc.first > 0 ? (uint32_t)sc.first : 0u, left = sc.first < 0 ? (uint32_t)-sc.first : 0u;
 #pragma unroll
     for (int k = 0; k < 8; k++) {
       const uint32_t rl = wlo(v[k].re), il = wlo(v[k].im), d = m - fx_code(rl, il) + right;
-      put(s, (i0 + k * ISTEP) * LS + l, swap, (int64_t)((uint64_t)fx_align(rl, (int32_t)whi(v[k].re), d) << left),
-          (int64_t)((uint64_t)fx_align(il, (int32_t)whi(v[k].im), d) << left));
+      x[k] = mk((int64_t)((uint64_t)fx_align(rl, (int32_t)whi(v[k].re), d) << left),
+                (int64_t)((uint64_t)fx_align(il, (int32_t)whi(v[k].im), d) << left));
     }
   } else {
     auto top = [&] {
@@ -215,31 +282,33 @@ __device__ __forceinline__ void pass(const PassParams<double>& p, cx<int64_t>* s
       L += fx_mag(whi(v[k].im), E - ((whi(v[k].im) >> 20) & 0x7ffu));
     }
     uint32_t any = 0;
-    sc = fx_schedule<LOGN>(64, fx_sum_bits(tile_sum<LOGC>(L, any, red[0], redm[1])));
+    sc = fx_schedule<LOGN>(64, fx_sum_bits(ti.sum(L, any, red[0], redm[1])));
     const uint32_t E2 = E + (uint32_t)sc.first;
     ex = (int32_t)E2 + off;
 #pragma unroll
     for (int k = 0; k < 8; k++) {
       const uint32_t rh = whi(v[k].re), ih = whi(v[k].im);
-      put(s, (i0 + k * ISTEP) * LS + l, swap, fx_from_double(rh, wlo(v[k].re), E2 - ((rh >> 20) & 0x7ffu)),
-          fx_from_double(ih, wlo(v[k].im), E2 - ((ih >> 20) & 0x7ffu)));
+      x[k] = mk(fx_from_double(rh, wlo(v[k].re), E2 - ((rh >> 20) & 0x7ffu)),
+                fx_from_double(ih, wlo(v[k].im), E2 - ((ih >> 20) & 0x7ffu)));
     }
   }
-  __syncthreads();
+  if (swap) exchange(x);
 
   // Transform (inverse, or the forward one of a kinetic pass), factors, transform (forward, or
   // the inverse one of a kinetic pass): one copy of the transform's code for both, because
   // the instruction cache holds little more (two copies waited on instruction fetches).
+  int spoil = 0;  // a factor that is not finite spoils its tile
   const bool t0 = kin || (f & F_IFFT), t1 = kin || (f & F_FFT), mid = ph || kin || (t0 && t1);
 #pragma unroll 1
   for (int it = 0; it < 2; it++) {
     if (it == 0 ? t0 : t1) {
-      fft<LOGN, LOGC, LS>(s, tw, sc, tid);
+      ti.fft(x, tw, sc);
       ex += sc.total - sc.first;
     }
     if (it == 1 || !mid) continue;
     // the factors of the middle of the pass, and the new bound for the transform after it
-    const int64_t line = CONTIG ? o0 + l : cb + l;
+    if (swap) exchange(x);
+    const int64_t line = ti.line(p.log_inner, tile);
     LineRec<double> rec = {};
     if (ph) rec = p.lines_phase[line];
     if (kin) rec = p.lines_kin[line];
@@ -254,52 +323,51 @@ __device__ __forceinline__ void pass(const PassParams<double>& p, cx<int64_t>* s
     const double* G0 = p.G[0][p.axis];
     const double* G1 = p.G[1][p.axis];
     int bad = sep && (rh & 0x7ff00000u) == 0x7ff00000u;
-    cx<int64_t> x[8];
-    uint32_t any = 0;
-    L = 0;
+    if (sep) {
 #pragma unroll
-    for (int k = 0; k < 8; k++) {
-      const int i = i0 + k * ISTEP;
-      x[k] = get(s, i * LS + l, swap);
-      if (sep) {
-        const FxRec a = A[i];
+      for (int k = 0; k < 8; k++) {
+        const FxRec a = A[ti.t + k * TL];
         bad |= a.bad;
         x[k] = fx_cmul(x[k], a);
         x[k] = fx_cmul(x[k], Lr);
       }
-      if (g0) x[k] = gauss_phase(x[k], rec.g[0] * G0[i], bad);
-      if (g1) x[k] = gauss_phase(x[k], rec.g[1] * G1[i], bad);
+    }
+    if (ph && p.ngauss > 0) {
+      ti.sync();
+#pragma unroll
+      for (int k = 0; k < 8; k++) ti.at(ti.t + k * TL) = x[k];
+      bad |= gauss_points(ti, g0 ? rec.g[0] : 0.0, g1 ? rec.g[1] : 0.0, G0, G1);
+#pragma unroll
+      for (int k = 0; k < 8; k++) x[k] = ti.at(ti.t + k * TL);
+    }
+    uint32_t any = 0;
+    L = 0;
+#pragma unroll
+    for (int k = 0; k < 8; k++) {
       const uint32_t ar = absh(x[k].re), ai = absh(x[k].im);
       any |= ar | ai;
       L += (ar >> 11) + (ai >> 11) + 2u;
     }
-    if (bad) spoil = 1;
-    swap = kin ? 1 : 0;
     if (t0 && t1) {
       // the transform before has changed the bounds: a new scale
-      const uint32_t Lm = tile_sum<LOGC>(L, any, red[1], redm[2]);
+      const uint32_t Lm = ti.sum(L, any, red[1], redm[2]);
       sc = fx_schedule<LOGN>(65 - __clz((int)any), fx_sum_bits(Lm));
       ex += sc.first;
 #pragma unroll
-      for (int k = 0; k < 8; k++)
-        put(s, (i0 + k * ISTEP) * LS + l, swap, shift_jam(x[k].re, sc.first), shift_jam(x[k].im, sc.first));
-    } else {
-#pragma unroll
-      for (int k = 0; k < 8; k++) s[(i0 + k * ISTEP) * LS + l] = x[k];
+      for (int k = 0; k < 8; k++) x[k] = mk(shift_jam(x[k].re, sc.first), shift_jam(x[k].im, sc.first));
     }
-    __syncthreads();
+    if (ph || kin) spoil = __syncthreads_or(bad);
+    swap = kin;
+    if (swap) exchange(x);
   }
+  if (swap) exchange(x);
   if (kin) ex -= p.g.ln[0] + p.g.ln[1] + p.g.ln[2];  // 1/N
   if (out_fx) {
     // each thread's eight points shifted up together, so that the code bits cost nothing of
     // their largest
-    cx<int64_t> x[8];
     uint32_t any = 0;
 #pragma unroll
-    for (int k = 0; k < 8; k++) {
-      x[k] = get(s, (i0 + k * ISTEP) * LS + l, swap);
-      any |= absh(x[k].re) | absh(x[k].im);
-    }
+    for (int k = 0; k < 8; k++) any |= absh(x[k].re) | absh(x[k].im);
     const uint32_t up = (uint32_t)max(__clz((int)any) - 1, 0);
     int32_t code = ex - (int32_t)up + kFxBias;
     if (code <= 0 || spoil) {
@@ -316,12 +384,11 @@ __device__ __forceinline__ void pass(const PassParams<double>& p, cx<int64_t>* s
   const bool chk = ex < 200 || ex > 1900;  // the range of a double may be left
 #pragma unroll
   for (int k = 0; k < 8; k++) {
-    const cx<int64_t> x = get(s, (i0 + k * ISTEP) * LS + l, swap);
     uint32_t rh, rl, ih, il;
-    fx_to_double(x.re, ex, rh, rl);
-    fx_to_double(x.im, ex, ih, il);
+    fx_to_double(x[k].re, ex, rh, rl);
+    fx_to_double(x[k].im, ex, ih, il);
     cx<double> y = mk(__hiloint2double((int)rh, (int)rl), __hiloint2double((int)ih, (int)il));
-    if (chk) y = scaled(x, ex - 1085);
+    if (chk) y = scaled(x[k], ex - 1085);
     if (spoil) y = mk(__longlong_as_double(0x7ff8000000000000ll), __longlong_as_double(0x7ff8000000000000ll));
     dst[k * step] = y;
   }
@@ -329,30 +396,18 @@ __device__ __forceinline__ void pass(const PassParams<double>& p, cx<int64_t>* s
 
 template <int LOGN, bool CONTIG>
 __device__ __forceinline__ void load(const cx<double>* in, int log_inner, int64_t tile, cx<double> (&v)[8]) {
-  using SH = FixShape<LOGN, CONTIG>;
-  constexpr int ISTEP = 256 >> SH::logC;
-  const int l = threadIdx.x & ((1 << SH::logC) - 1), i0 = threadIdx.x >> SH::logC;
-  int64_t base, es;
-  if (CONTIG) {
-    base = (((tile << SH::logC) + l) << SH::logn) + i0;
-    es = 1;
-  } else {
-    const int tpo = log_inner - SH::logC;
-    const int64_t o0 = tile >> tpo, cb = (tile & ((int64_t(1) << tpo) - 1)) << SH::logC;
-    es = int64_t(1) << log_inner;
-    base = (((o0 << SH::logn) + i0) << log_inner) + cb + l;
-  }
-  const cx<double>* q = in + base;
+  int64_t step;
+  const cx<double>* q = in + Tile<LOGN, CONTIG>(nullptr).base(log_inner, tile, step);
 #pragma unroll
-  for (int k = 0; k < 8; k++) v[k] = q[k * es * ISTEP];
+  for (int k = 0; k < 8; k++) v[k] = q[k * step];
 }
 
 template <int LOGN, bool CONTIG>
-__global__ void __launch_bounds__(256, 4) k_pass_fx(const PassParams<double> p) {
+__global__ void __launch_bounds__(256, 3) k_pass_fx(const PassParams<double> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cx<double> v[8];
   load<LOGN, CONTIG>(p.in, p.log_inner, blockIdx.x, v);
-  pass<LOGN, CONTIG>(p, reinterpret_cast<cx<int64_t>*>(smem_raw), blockIdx.x, v);
+  pass<LOGN, CONTIG>(p, smem_raw, blockIdx.x, v);
 }
 
 }  // namespace fxp

@@ -68,6 +68,8 @@ __host__ __device__ constexpr int wp_stage_tw_offset(int logn, int logNs) {
 // 193 -> 129 us.
 constexpr int kFixedLogMin = 5, kFixedLogMax = 11;
 constexpr int kFixedObsLogMin = 6, kFixedObsLogMax = 10;
+// Shared memory of a complex128 tile in fixed point (2048 points, one place in eight left free).
+constexpr size_t kFxTileBytes = 2304 * 16;
 constexpr int kRes1dLogMin = 8, kRes1dLogMax = 14;  // fixed-length resident lines: n = 256..16384
 
 // A table factor as one 16-byte record: the value for FP64 and float-float, the high
@@ -209,7 +211,6 @@ struct AxisTab {
   void* W2s;                  // complex64, n = 64 or 128: two-stage twiddle records (wp_pass2s.cuh)
   // complex128: the fixed-point factors (wp_fx.h). Stage twiddles (at the offsets of Wst),
   // kinetic factors without the 1/N of axis 0, and the potential phase factors of the step.
-  FxRec* Wfx;
   FxRec* Kfx_full;
   FxRec* Kfx_half;
   FxRec* Pfx;
@@ -266,7 +267,6 @@ struct PassParams {
   const void* W256;        // two-stage 256-point kernels: twiddle records of the pass axis, or NULL
   const void* W2s;         // two-stage 64- and 128-point kernels: twiddle records, or NULL
   // complex128: the pass axis's fixed-point factors (AxisTab)
-  const FxRec* Wfx;
   const FxRec* Pfx;
   const FxRec* Kfx;
   const FxRec* Kfx_half;

@@ -1207,7 +1207,9 @@ __device__ __forceinline__ void pass_body(const PassParams<T>& p, const SH& sh, 
 // The complex128 passes in fixed point (wp_fx_pass.cuh).
 namespace fxp {
 template <int LOGN, bool CONTIG>
-__device__ __forceinline__ void pass(const PassParams<double>& p, cx<int64_t>* s, int64_t tile, cx<double> (&v)[8]);
+__device__ __forceinline__ void load(const cx<double>* in, int log_inner, int64_t tile, cx<double> (&v)[8]);
+template <int LOGN, bool CONTIG>
+__device__ __forceinline__ void pass(const PassParams<double>& p, void* smem, int64_t tile, cx<double> (&v)[8]);
 }  // namespace fxp
 
 // E elements per thread; the block has at most 32 E threads, so a tile holds at most
@@ -1239,7 +1241,9 @@ __device__ __forceinline__ void pass_batch_body(const PassParams<T>* __restrict_
   // are issued before the parameter copy and the two latencies overlap
   [[maybe_unused]] cx<T> v[8];
   [[maybe_unused]] int vl = 0, vi0 = 0;
-  if constexpr (LOGN > 0) {
+  if constexpr (LOGN > 0 && std::is_same<T, double>::value) {
+    fxp::load<LOGN, CONTIG>(params[inst].in, params[inst].log_inner, tile, v);
+  } else if constexpr (LOGN > 0) {
     using SH = FixShape<LOGN, CONTIG>;
     constexpr int ISTEP = 256 >> SH::logC;
     const cx<T>* in = params[inst].in;
@@ -1279,7 +1283,7 @@ __device__ __forceinline__ void pass_batch_body(const PassParams<T>* __restrict_
   __syncthreads();
   cx<T>* s = reinterpret_cast<cx<T>*>(smem_raw);
   if constexpr (LOGN > 0 && std::is_same<T, double>::value) {
-    fxp::pass<LOGN, CONTIG>(p, reinterpret_cast<cx<int64_t>*>(smem_raw), tile, v);
+    fxp::pass<LOGN, CONTIG>(p, smem_raw, tile, v);
   } else if constexpr (LOGN > 0) {
     using SH = FixShape<LOGN, CONTIG>;
     constexpr int ISTEP = 256 >> SH::logC;
