@@ -903,10 +903,10 @@ template <class T>
 wp_status momentum_and_reduce(wp_handle* h) {
   wp_status st;
   const int nd = h->ndim;
-  if ((st = run_pass<T>(h, nd - 1, F_FFT | (nd == 3 ? F_OUT_FX : 0u), h->state, h->scratch)) != WP_OK) return st;
+  if ((st = run_pass<T>(h, nd - 1, F_FFT | F_OUT_FX, h->state, h->scratch)) != WP_OK) return st;
   if (nd == 3)
-    if ((st = run_pass<T>(h, 1, F_FFT | F_IN_FX, h->scratch, h->scratch)) != WP_OK) return st;
-  if ((st = run_pass<T>(h, 0, F_FFT | F_OBS_MOM | F_NO_STORE, h->scratch, h->scratch, h->part_mom)) != WP_OK)
+    if ((st = run_pass<T>(h, 1, F_FFT | F_IN_FX | F_OUT_FX, h->scratch, h->scratch)) != WP_OK) return st;
+  if ((st = run_pass<T>(h, 0, F_FFT | F_OBS_MOM | F_NO_STORE | F_IN_FX, h->scratch, h->scratch, h->part_mom)) != WP_OK)
     return st;
   ReduceParams r{};
   r.pos = h->part_pos;
@@ -975,38 +975,36 @@ wp_status chunk_seq(wp_handle* h, int64_t m, bool obs_end) {
   }
   void* S = h->state;
   const int Z = nd - 1;
-  // between the passes of the chunk a complex128 state is in fixed point (fx_state); a pass
-  // that forms observable sums is FP64 and reads doubles
+  // between the passes of the chunk a complex128 state is in fixed point (fx_state)
   constexpr uint32_t FX = F_IN_FX | F_OUT_FX;
-  auto middle = [&](int khalf, bool to_fx) -> wp_status {
+  auto middle = [&](int khalf) -> wp_status {
     wp_status s2;
-    const uint32_t last = F_IN_FX | (to_fx ? F_OUT_FX : 0u);
     if (nd == 3)
       if ((s2 = run_pass<T>(h, 1, F_FFT | FX, S, S)) != WP_OK) return s2;
-    if ((s2 = run_pass<T>(h, 0, F_KIN | (nd == 3 ? FX : last), S, S, nullptr, khalf)) != WP_OK) return s2;
+    if ((s2 = run_pass<T>(h, 0, F_KIN | FX, S, S, nullptr, khalf)) != WP_OK) return s2;
     if (nd == 3)
-      if ((s2 = run_pass<T>(h, 1, F_IFFT | last, S, S)) != WP_OK) return s2;
+      if ((s2 = run_pass<T>(h, 1, F_IFFT | FX, S, S)) != WP_OK) return s2;
     return WP_OK;
   };
-  const uint32_t obsf = obs_end ? (F_OBS_POS | (h->pb.autocorr ? F_AUTOCORR : 0u)) : F_IN_FX;
+  const uint32_t obsf = F_IN_FX | (obs_end ? (F_OBS_POS | (h->pb.autocorr ? F_AUTOCORR : 0u)) : 0u);
   // the tables of step k + 1 are formed beside the strided passes of step k
   if (h->pb.order == WP_ORDER_VKV) {
     if ((st = run_prep<T>(h, 0, 0.0, 0.5 * dt, true)) != WP_OK) return st;
     if ((st = run_pass<T>(h, Z, F_PHASE | F_FFT | F_OUT_FX, S, S)) != WP_OK) return st;
     for (int64_t k = 1; k < m; k++) {
       if ((st = fork_tables<T>(h, 1, 0.0, dt, true)) != WP_OK) return st;
-      if ((st = middle(0, true)) != WP_OK) return st;
+      if ((st = middle(0)) != WP_OK) return st;
       if ((st = join_tables(h)) != WP_OK) return st;
       if ((st = run_pass<T>(h, Z, F_IFFT | F_PHASE | F_FFT | FX, S, S)) != WP_OK) return st;
     }
     if ((st = fork_tables<T>(h, 1, 0.0, 0.5 * dt, true)) != WP_OK) return st;
-    if ((st = middle(0, !obs_end)) != WP_OK) return st;
+    if ((st = middle(0)) != WP_OK) return st;
     if ((st = join_tables(h)) != WP_OK) return st;
     if ((st = run_pass<T>(h, Z, F_IFFT | F_PHASE | obsf, S, S, h->part_pos)) != WP_OK) return st;
   } else {
     if ((st = run_pass<T>(h, Z, F_FFT | F_OUT_FX, S, S)) != WP_OK) return st;
     if ((st = fork_tables<T>(h, 0, 0.5 * dt, dt, true)) != WP_OK) return st;
-    if ((st = middle(1, true)) != WP_OK) return st;
+    if ((st = middle(1)) != WP_OK) return st;
     for (int64_t k = 0; k < m; k++) {
       if ((st = join_tables(h)) != WP_OK) return st;
       if ((st = run_pass<T>(h, Z, F_IFFT | F_PHASE | F_FFT | FX, S, S)) != WP_OK) return st;
@@ -1015,7 +1013,7 @@ wp_status chunk_seq(wp_handle* h, int64_t m, bool obs_end) {
       } else {
         if ((st = fork_tables<T>(h, 1, 0.0, 0.0, false)) != WP_OK) return st;
       }
-      if ((st = middle(k == m - 1 ? 1 : 0, k < m - 1 || !obs_end)) != WP_OK) return st;
+      if ((st = middle(k == m - 1 ? 1 : 0)) != WP_OK) return st;
     }
     if ((st = join_tables(h)) != WP_OK) return st;
     if ((st = run_pass<T>(h, Z, F_IFFT | obsf, S, S, h->part_pos)) != WP_OK) return st;

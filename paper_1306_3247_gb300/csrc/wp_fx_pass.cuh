@@ -1,8 +1,8 @@
 // Passes of the complex128 form in 64-bit fixed point (wp_fx.h): a tile is held as integers
 // with one exponent through the transforms and factors of the pass. Tiles, stage plan and
 // thread mapping are those of the fixed-shape kernels of wp_kernels.cuh (2048 points, 256
-// threads, n = 32..2048, the lengths whose stages unroll); the passes that form observable
-// sums or apply a grid potential stay in FP64.
+// threads, n = 32..2048, the lengths whose stages unroll); those that form observable sums
+// add them up in FP64 from the results; passes that apply a grid potential stay in FP64.
 //
 // Bound by the integer pipe (64 lanes per clock; ncu on 256^3: 61 % busy over the launch,
 // FP64 before 92 %) and by instruction issue (62 %). Measured on the 256^3 barrier, CUDA
@@ -196,9 +196,11 @@ __device__ __noinline__ int gauss_points(TI ti, double a0, double a1, const doub
   return bad;
 }
 
-// v: the thread's points, loaded by the caller.
-template <int LOGN, bool CONTIG>
-__device__ __forceinline__ void pass(const PassParams<double>& p, void* smem, int64_t tile, cx<double> (&v)[8]) {
+// v: the thread's points, loaded by the caller. OBS: v returns the pass's results as doubles
+// for the sums, unless the tile is empty or not finite: then its row of the sums is written
+// here and the result is false.
+template <int LOGN, bool CONTIG, bool OBS>
+__device__ __forceinline__ bool pass(const PassParams<double>& p, void* smem, int64_t tile, cx<double> (&v)[8]) {
   using TI = Tile<LOGN, CONTIG>;
   constexpr int TL = TI::TL;
   __shared__ uint32_t red[2][256];
@@ -225,7 +227,10 @@ __device__ __forceinline__ void pass(const PassParams<double>& p, void* smem, in
   auto fill = [&](bool finite) {
     const double z = finite ? 0.0 : (out_fx ? __longlong_as_double(63) : __longlong_as_double(0x7ff8000000000000ll));
 #pragma unroll
-    for (int k = 0; k < 8; k++) dst[k * step] = mk(z, z);
+    for (int k = 0; k < 8; k++)
+      if (!OBS || !(f & F_NO_STORE)) dst[k * step] = mk(z, z);
+    if (OBS && tid < NQ) p.partials[tile * NQ + tid] = z;
+    return false;
   };
   FxSchedule sc;
   int32_t ex;
@@ -362,7 +367,7 @@ __device__ __forceinline__ void pass(const PassParams<double>& p, void* smem, in
   }
   if (swap) exchange(x);
   if (kin) ex -= p.g.ln[0] + p.g.ln[1] + p.g.ln[2];  // 1/N
-  if (out_fx) {
+  if (!OBS && out_fx) {
     // each thread's eight points shifted up together, so that the code bits cost nothing of
     // their largest
     uint32_t any = 0;
@@ -379,7 +384,7 @@ __device__ __forceinline__ void pass(const PassParams<double>& p, void* smem, in
       const uint32_t rl = ((uint32_t)re & ~63u) | ((uint32_t)code >> 6), il = ((uint32_t)im & ~63u) | ((uint32_t)code & 63u);
       dst[k * step] = mk(__hiloint2double((int)(re >> 32), (int)rl), __hiloint2double((int)(im >> 32), (int)il));
     }
-    return;
+    return true;
   }
   const bool chk = ex < 200 || ex > 1900;  // the range of a double may be left
 #pragma unroll
@@ -390,7 +395,97 @@ __device__ __forceinline__ void pass(const PassParams<double>& p, void* smem, in
     cx<double> y = mk(__hiloint2double((int)rh, (int)rl), __hiloint2double((int)ih, (int)il));
     if (chk) y = scaled(x[k], ex - 1085);
     if (spoil) y = mk(__longlong_as_double(0x7ff8000000000000ll), __longlong_as_double(0x7ff8000000000000ll));
-    dst[k * step] = y;
+    if (!OBS || !(f & F_NO_STORE)) dst[k * step] = y;
+    if (OBS) v[k] = y;
+  }
+  return true;
+}
+
+// The tile's row of the observable sums (obs_line_row's line sums), from the thread's points
+// v: position sums on a contiguous axis, momentum sums on a strided one. Every FP64
+// instruction counts (one per 19 clocks and SM): the threads' eight sums cross shared memory
+// once, and each warp adds up one of the eight, 8 + log2(32 / C) additions against the 40
+// of a shuffle tree over all eight.
+template <int LOGN, bool CONTIG>
+__device__ __forceinline__ void obs_sums(const PassParams<double>& p, void* smem, int64_t tile, const cx<double> (&v)[8]) {
+  using TI = Tile<LOGN, CONTIG>;
+  constexpr int C = TI::C, CW = C < 32 ? C : 32;
+  __shared__ double red[C][NQ];
+  const TI ti(smem);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  double q[8];
+#pragma unroll
+  for (int j = 0; j < 8; j++) q[j] = 0.0;
+  if constexpr (CONTIG) {
+    const double* G0 = p.G[0][p.axis];
+    const double* G1 = p.G[1][p.axis];
+    int64_t step;
+    const int64_t base = ti.base(p.log_inner, tile, step);
+#pragma unroll
+    for (int k = 0; k < 8; k++) {
+      const int i = ti.t + k * TI::TL;
+      const double rho = norm2(v[k]);
+      const cx<double> xx = p.Ox[i];
+      q[0] += rho;
+      q[1] = madd(xx.re, rho, q[1]);
+      q[2] = madd(xx.im, rho, q[2]);
+      q[3] = madd(p.AT[i], rho, q[3]);
+      if (p.ngauss > 0) q[4] = madd(G0[i], rho, q[4]);
+      if (p.ngauss > 1) q[5] = madd(G1[i], rho, q[5]);
+      if (p.flags & F_AUTOCORR) {
+        const cx<double> c = cmulc(v[k], p.psi0[base + k * step]);
+        q[6] += c.re;
+        q[7] += c.im;
+      }
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < 8; k++) {
+      const double rho = norm2(v[k]);
+      const cx<double> kk = p.Ok[ti.t + k * TI::TL];
+      q[0] += rho;
+      q[1] = madd(kk.re, rho, q[1]);
+      q[2] = madd(kk.im, rho, q[2]);
+    }
+  }
+  constexpr int ROW = 256 + 16;  // one place in 16 left free against bank conflicts
+  double* sc = reinterpret_cast<double*>(smem);
+  const int e = ti.t * C + ti.l;
+  __syncthreads();  // the tile is free now
+#pragma unroll
+  for (int j = 0; j < 8; j++) sc[j * ROW + e + (e >> 4)] = q[j];
+  __syncthreads();
+  double a[2] = {0.0, 0.0};
+#pragma unroll
+  for (int m = 0; m < 8; m++) {
+    const int r = lane + 32 * m;
+    a[C > 32 ? m & 1 : 0] += sc[warp * ROW + r + (r >> 4)];
+  }
+#pragma unroll
+  for (int o = C; o < 32; o <<= 1) a[0] += __shfl_xor_sync(0xffffffffu, a[0], o);
+  if (lane < CW) {
+    red[lane][warp] = a[0];
+    if (C > 32) red[(lane + 32) & (C - 1)][warp] = a[1];
+  }
+  __syncthreads();
+  double lt[8];
+  if (tid < C) {
+#pragma unroll
+    for (int j = 0; j < 8; j++) lt[j] = red[tid][j];
+    int gi[3];
+    const int tpo = p.log_inner - TI::LOGC;
+    if (CONTIG)
+      grid_index(p.g, p.axis, (tile << TI::LOGC) + tid, 0, 0, gi);
+    else
+      grid_index(p.g, p.axis, tile >> tpo, ((tile & ((int64_t(1) << tpo) - 1)) << TI::LOGC) + tid, 0, gi);
+    obs_line_row(p, lt, gi, red[tid]);
+  }
+  __syncthreads();
+  if (tid < NQ) {
+    double sum = 0.0;
+#pragma unroll 8
+    for (int l = 0; l < C; l++) sum += red[l][tid];
+    p.partials[tile * NQ + tid] = sum;
   }
 }
 
@@ -402,12 +497,27 @@ __device__ __forceinline__ void load(const cx<double>* in, int log_inner, int64_
   for (int k = 0; k < 8; k++) v[k] = q[k * step];
 }
 
+// Three blocks per SM (80 registers); with four (64, and x spilled) the step at 256^3 takes
+// 994 us against 960, at 1024 x 1024 80 against 74.
 template <int LOGN, bool CONTIG>
 __global__ void __launch_bounds__(256, 3) k_pass_fx(const PassParams<double> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cx<double> v[8];
   load<LOGN, CONTIG>(p.in, p.log_inner, blockIdx.x, v);
-  pass<LOGN, CONTIG>(p, smem_raw, blockIdx.x, v);
+  pass<LOGN, CONTIG, false>(p, smem_raw, blockIdx.x, v);
+}
+
+// With the observable sums of the tile. A record of the 256^3 barrier (its three or four
+// passes, with the FP64 butterflies before) cost 1.5 + 1.1 ms for the two passes that form
+// sums; the run of 20 steps and 2 records takes 20.6 ms with these, 23.0 before.
+template <int LOGN, bool CONTIG>
+__global__ void __launch_bounds__(256, 3) k_pass_fx_obs(const PassParams<double> p) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  cx<double> v[8];
+  load<LOGN, CONTIG>(p.in, p.log_inner, blockIdx.x, v);
+  if ((p.flags & (F_IFFT | F_PHASE | F_FFT | F_KIN)) || !(p.flags & F_NO_STORE))
+    if (!pass<LOGN, CONTIG, true>(p, smem_raw, blockIdx.x, v)) return;
+  obs_sums<LOGN, CONTIG>(p, smem_raw, blockIdx.x, v);
 }
 
 }  // namespace fxp

@@ -60,8 +60,8 @@ __host__ __device__ constexpr int wp_stage_tw_offset(int logn, int logNs) {
   }
   return off;
 }
-// Fixed-size pass kernels: n = 32..2048; those that also form observable sums or apply a grid
-// potential, n = 64..1024.
+// Fixed-size pass kernels: n = 32..2048; those that apply a grid potential, and the complex64
+// and float-float ones that also form observable sums, n = 64..1024.
 // Measured a step at 32 and 2048 points, run-time kernels -> these: complex128 2048 x 1024
 // 559 -> 164 us, 32 x 64 x 64 82 -> 43 us; complex64 2048 x 1024 115 -> 51 us,
 // 2048 x 512 x 64 3668 -> 1810 us, 32 x 64 x 128 24.6 -> 17.2 us; float-float 2048 x 1024

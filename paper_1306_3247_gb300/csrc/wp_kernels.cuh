@@ -1208,8 +1208,8 @@ __device__ __forceinline__ void pass_body(const PassParams<T>& p, const SH& sh, 
 namespace fxp {
 template <int LOGN, bool CONTIG>
 __device__ __forceinline__ void load(const cx<double>* in, int log_inner, int64_t tile, cx<double> (&v)[8]);
-template <int LOGN, bool CONTIG>
-__device__ __forceinline__ void pass(const PassParams<double>& p, void* smem, int64_t tile, cx<double> (&v)[8]);
+template <int LOGN, bool CONTIG, bool OBS>
+__device__ __forceinline__ bool pass(const PassParams<double>& p, void* smem, int64_t tile, cx<double> (&v)[8]);
 }  // namespace fxp
 
 // E elements per thread; the block has at most 32 E threads, so a tile holds at most
@@ -1283,7 +1283,7 @@ __device__ __forceinline__ void pass_batch_body(const PassParams<T>* __restrict_
   __syncthreads();
   cx<T>* s = reinterpret_cast<cx<T>*>(smem_raw);
   if constexpr (LOGN > 0 && std::is_same<T, double>::value) {
-    fxp::pass<LOGN, CONTIG>(p, smem_raw, tile, v);
+    fxp::pass<LOGN, CONTIG, false>(p, smem_raw, tile, v);
   } else if constexpr (LOGN > 0) {
     using SH = FixShape<LOGN, CONTIG>;
     constexpr int ISTEP = 256 >> SH::logC;

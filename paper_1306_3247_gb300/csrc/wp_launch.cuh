@@ -36,7 +36,7 @@ int res1d_smem_limit_set(size_t smem) {
 }
 
 // p.fixed selects the fixed-size kernel (n = 32..2048, 2048-element tiles, 256 threads),
-// with partial sums (n = 64..1024) when they are positions on the contiguous axis or momenta on a
+// with partial sums (complex64 and float-float: n = 64..1024) when they are positions on the contiguous axis or momenta on a
 // strided one; otherwise p.ept selects the run-time variant (8 elements per thread: <= 256 threads;
 // 16: <= 512).
 template <class T>
@@ -56,14 +56,14 @@ int launch_pass(const PassParams<T>& p, int64_t ntiles, size_t smem, void* strea
     const bool contig = p.log_inner == 0;
     // a static grid potential enters the potential phase and the position sums
     const bool use_grid = (p.grid_rec && (p.flags & F_PHASE)) || (p.grid_v && (p.flags & F_OBS_POS));
-    const bool sums = p.logn >= kFixedObsLogMin && p.logn <= kFixedObsLogMax;  // lengths with OBS and GRID kernels
+    const bool sums = p.logn >= kFixedObsLogMin && p.logn <= kFixedObsLogMax;  // lengths of all kernels
     if (use_grid) {
       if (sums && contig && !(p.flags & F_OBS_MOM))
         return obs ? launch_fixed_grid_obs<T>(p, grid.x, smem, stream) : launch_fixed_grid<T>(p, grid.x, smem, stream);
     } else {
       if (!obs) return launch_fixed<T>(p, grid.x, smem, stream);
       // the fixed variant sums positions on the contiguous axis, momenta on a strided one
-      if (sums && ((contig && !(p.flags & F_OBS_MOM)) || (!contig && !(p.flags & F_OBS_POS))))
+      if ((sums || std::is_same<T, double>::value) && ((contig && !(p.flags & F_OBS_MOM)) || (!contig && !(p.flags & F_OBS_POS))))
         return launch_fixed_obs<T>(p, grid.x, smem, stream);
     }
   }
