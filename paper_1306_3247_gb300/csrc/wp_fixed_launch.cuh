@@ -35,10 +35,10 @@ constexpr int kLogMax = kAllLengths<T, OBS, GRID> ? kFixedLogMax : kFixedObsLogM
 template <class T, bool OBS, bool GRID, int LOGN>
 cudaError_t launch_n(const PassParams<T>& p, unsigned ntiles, size_t smem, cudaStream_t st) {
   if (p.log_inner == 0) {
-    kernel_of<T, LOGN, true, OBS, GRID>()<<<ntiles, 256, smem, st>>>(p);
+    launch_dep(kernel_of<T, LOGN, true, OBS, GRID>(), ntiles, 256, smem, st, p);
   } else {
     if constexpr (GRID) return cudaErrorInvalidConfiguration;
-    else kernel_of<T, LOGN, false, OBS, false>()<<<ntiles, 256, smem, st>>>(p);
+    else launch_dep(kernel_of<T, LOGN, false, OBS, false>(), ntiles, 256, smem, st, p);
   }
   return cudaGetLastError();
 }

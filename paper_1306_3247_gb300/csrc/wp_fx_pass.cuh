@@ -502,6 +502,7 @@ __device__ __forceinline__ void load(const cx<double>* in, int log_inner, int64_
 template <int LOGN, bool CONTIG>
 __global__ void __launch_bounds__(256, 3) k_pass_fx(const PassParams<double> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  pass_begin();
   cx<double> v[8];
   load<LOGN, CONTIG>(p.in, p.log_inner, blockIdx.x, v);
   pass<LOGN, CONTIG, false>(p, smem_raw, blockIdx.x, v);
@@ -509,10 +510,11 @@ __global__ void __launch_bounds__(256, 3) k_pass_fx(const PassParams<double> p) 
 
 // With the observable sums of the tile. A record of the 256^3 barrier (its three or four
 // passes, with the FP64 butterflies before) cost 1.5 + 1.1 ms for the two passes that form
-// sums; the run of 20 steps and 2 records takes 20.6 ms with these, 23.0 before.
+// sums; the run of 20 steps and 2 records takes 20.6 ms with these, about 23 before.
 template <int LOGN, bool CONTIG>
 __global__ void __launch_bounds__(256, 3) k_pass_fx_obs(const PassParams<double> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  pass_begin();
   cx<double> v[8];
   load<LOGN, CONTIG>(p.in, p.log_inner, blockIdx.x, v);
   if ((p.flags & (F_IFFT | F_PHASE | F_FFT | F_KIN)) || !(p.flags & F_NO_STORE))

@@ -14,8 +14,8 @@ int launch_reduce_rows(ReduceParams& p, void* stream) {
   int64_t R = (rows + 303) / 304;
   if (R < 256) R = 256;
   const unsigned nb = (unsigned)((rows + R - 1) / R);
-  k_reduce_rows<<<dim3(nb, 2), 256, 0, (cudaStream_t)stream>>>(const_cast<double*>(p.pos), p.npos,
-                                                                 const_cast<double*>(p.mom), p.nmom, R);
+  launch_dep(k_reduce_rows, dim3(nb, 2), 256, 0, (cudaStream_t)stream, const_cast<double*>(p.pos), p.npos,
+             const_cast<double*>(p.mom), p.nmom, R);
   p.npos = (p.npos + R - 1) / R;
   p.nmom = (p.nmom + R - 1) / R;
   p.pos_stride = p.mom_stride = R;
@@ -23,12 +23,12 @@ int launch_reduce_rows(ReduceParams& p, void* stream) {
 }
 
 int launch_reduce(const ReduceParams& p, void* stream) {
-  k_reduce<<<1, 256, 0, (cudaStream_t)stream>>>(p);
+  launch_dep(k_reduce, 1, 256, 0, (cudaStream_t)stream, p);
   return cuda_status(cudaGetLastError());
 }
 
 int launch_set_step(Ctrl* ctrl, int64_t step, void* stream) {
-  k_set_step<<<1, 1, 0, (cudaStream_t)stream>>>(ctrl, step);
+  launch_dep(k_set_step, 1, 1, 0, (cudaStream_t)stream, ctrl, step);
   return cuda_status(cudaGetLastError());
 }
 

@@ -69,14 +69,14 @@ int launch_pass(const PassParams<T>& p, int64_t ntiles, size_t smem, void* strea
   }
   if (p.ept == 8 && p.nthreads <= 256) {
     if (obs)
-      k_pass<T, 8, true><<<grid, block, smem, st>>>(p);
+      launch_dep(k_pass<T, 8, true>, grid, block, smem, st, p);
     else
-      k_pass<T, 8, false><<<grid, block, smem, st>>>(p);
+      launch_dep(k_pass<T, 8, false>, grid, block, smem, st, p);
   } else if (p.ept == 16 && p.nthreads <= 512) {
     if (obs)
-      k_pass<T, 16, true><<<grid, block, smem, st>>>(p);
+      launch_dep(k_pass<T, 16, true>, grid, block, smem, st, p);
     else
-      k_pass<T, 16, false><<<grid, block, smem, st>>>(p);
+      launch_dep(k_pass<T, 16, false>, grid, block, smem, st, p);
   } else {
     return (int)cudaErrorInvalidConfiguration;
   }
@@ -92,7 +92,7 @@ int launch_prep(const PrepParams<T>& p, int ngauss, void* stream) {
   int64_t blocks = (nall + 63) / 64;
   if (blocks < 1) blocks = 1;
   if (blocks > 512) blocks = 512;
-  k_prep<T><<<(unsigned)blocks, 64, 0, (cudaStream_t)stream>>>(p);
+  launch_dep(k_prep<T>, (unsigned)blocks, 64, 0, (cudaStream_t)stream, p);
   return cuda_status(cudaGetLastError());
 }
 
@@ -157,7 +157,7 @@ template <class T>
 int launch_lines(const LinesParams<T>& p, void* stream) {
   int64_t blocks = (p.nlines + 255) / 256;
   if (blocks > 4096) blocks = 4096;
-  if (blocks > 0) k_lines<T><<<(unsigned)blocks, 256, 0, (cudaStream_t)stream>>>(p);
+  if (blocks > 0) launch_dep(k_lines<T>, (unsigned)blocks, 256, 0, (cudaStream_t)stream, p);
   return cuda_status(cudaGetLastError());
 }
 

@@ -723,6 +723,7 @@ template <class T, int LOGN, int LOGR>
 __global__ void __launch_bounds__(Shape<T, LOGN, LOGR>::NT + Shape<T, LOGN, LOGR>::TW)
     k_line(const Res1dParams<T> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  pass_begin();
   body<T, LOGN, LOGR, false>(p, smem_raw);
 }
 

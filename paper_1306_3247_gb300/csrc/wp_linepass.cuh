@@ -95,6 +95,7 @@ __global__ void __launch_bounds__(Shape<T, LOGN, CONTIG, WIDE>::NT, Shape<T, LOG
   using SH = Shape<T, LOGN, CONTIG, WIDE>;
   constexpr int TL = SH::TL;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  pass_begin();
   Tile<T, LOGN, CONTIG, WIDE> tile{reinterpret_cast<cx<T>*>(smem_raw), 0, 0};
   int64_t base, es, line;
   if constexpr (CONTIG) {
@@ -180,7 +181,7 @@ cudaError_t go(const PassParams<T>& p, cudaStream_t st) {
   int lntot = 0;
   for (int d = 0; d < p.g.ndim; d++) lntot += p.g.ln[d];
   const unsigned blocks = (unsigned)((int64_t(1) << (lntot - LOGN)) / SH::C);
-  kern<<<blocks, SH::NT, SH::SMEM, st>>>(p);
+  launch_dep(kern, blocks, SH::NT, SH::SMEM, st, p);
   return cudaGetLastError();
 }
 

@@ -532,6 +532,7 @@ __device__ __forceinline__ void strided_body(const PassParams<T>& p, int64_t o, 
 template <class T, int NG, bool SEP, bool OBS = false>
 __global__ void __launch_bounds__(threads_of<T>(), Shape<T>::kMinBlocks) k_pass256_contig(const PassParams<T> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  pass_begin();
   // the line loads are issued before the twiddle table's (their latencies overlap)
   cx<T> v[16];
   contig_load(p.in, blockIdx.x, v);
@@ -541,6 +542,7 @@ __global__ void __launch_bounds__(threads_of<T>(), Shape<T>::kMinBlocks) k_pass2
 template <class T, bool KIN, bool OBS = false>
 __global__ void __launch_bounds__(threads_of<T>(), Shape<T>::kMinBlocks) k_pass256_strided(const PassParams<T> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  pass_begin();
   int64_t o, cb;
   strided_origin<T>(p.log_inner, blockIdx.x, o, cb);
   float4 ld[Stage<T>::Q];

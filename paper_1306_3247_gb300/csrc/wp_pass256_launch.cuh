@@ -55,16 +55,16 @@ void launch_contig_ng(const PassParams<T>& p, unsigned blocks, cudaStream_t st) 
   if constexpr (std::is_same<T, float>::value) {
     if (p.flags & F_OBS_POS) {
       if (p.sep)
-        p256::k_pass256_contig<T, NG, true, true><<<blocks, nt, p256::kSmem, st>>>(p);
+        launch_dep(p256::k_pass256_contig<T, NG, true, true>, blocks, nt, p256::kSmem, st, p);
       else
-        p256::k_pass256_contig<T, NG, false, true><<<blocks, nt, p256::kSmem, st>>>(p);
+        launch_dep(p256::k_pass256_contig<T, NG, false, true>, blocks, nt, p256::kSmem, st, p);
       return;
     }
   }
   if (p.sep)
-    p256::k_pass256_contig<T, NG, true><<<blocks, nt, p256::kSmem, st>>>(p);
+    launch_dep(p256::k_pass256_contig<T, NG, true>, blocks, nt, p256::kSmem, st, p);
   else
-    p256::k_pass256_contig<T, NG, false><<<blocks, nt, p256::kSmem, st>>>(p);
+    launch_dep(p256::k_pass256_contig<T, NG, false>, blocks, nt, p256::kSmem, st, p);
 }
 
 // Tensor maps of the TMA-staged strided kernel: the state seen as rows of 2^log_inner
@@ -132,22 +132,22 @@ int launch(const PassParams<T>& p, void* stream) {
       alignas(64) CUtensorMap tin, tout;
       if (enc && tile_map(enc, p.in, p.log_inner, lntot, &tin) && tile_map(enc, p.out, p.log_inner, lntot, &tout)) {
         if (p.flags & F_KIN)
-          p256::k_pass256_strided_tma<true><<<blocks, 256, p256::kTmaSmem, st>>>(p, tin, tout);
+          launch_dep(p256::k_pass256_strided_tma<true>, blocks, 256, p256::kTmaSmem, st, p, tin, tout);
         else if (p.flags & F_OBS_MOM)
-          p256::k_pass256_strided_tma<false, true><<<blocks, 256, p256::kTmaSmem, st>>>(p, tin, tout);
+          launch_dep(p256::k_pass256_strided_tma<false, true>, blocks, 256, p256::kTmaSmem, st, p, tin, tout);
         else
-          p256::k_pass256_strided_tma<false><<<blocks, 256, p256::kTmaSmem, st>>>(p, tin, tout);
+          launch_dep(p256::k_pass256_strided_tma<false>, blocks, 256, p256::kTmaSmem, st, p, tin, tout);
         done = true;
       }
     }
     if (!done) {
       constexpr unsigned nt = p256::threads_of<T>();
       if (p.flags & F_KIN)
-        p256::k_pass256_strided<T, true><<<blocks, nt, p256::kSmem, st>>>(p);
+        launch_dep(p256::k_pass256_strided<T, true>, blocks, nt, p256::kSmem, st, p);
       else if (std::is_same<T, float>::value && (p.flags & F_OBS_MOM))
-        p256::k_pass256_strided<T, false, std::is_same<T, float>::value><<<blocks, nt, p256::kSmem, st>>>(p);
+        launch_dep(p256::k_pass256_strided<T, false, std::is_same<T, float>::value>, blocks, nt, p256::kSmem, st, p);
       else
-        p256::k_pass256_strided<T, false><<<blocks, nt, p256::kSmem, st>>>(p);
+        launch_dep(p256::k_pass256_strided<T, false>, blocks, nt, p256::kSmem, st, p);
     }
   }
   const cudaError_t e = cudaGetLastError();

@@ -78,6 +78,7 @@ __global__ void __launch_bounds__(256, Shape<float>::kMinBlocks)
     k_pass256_strided_tma(const PassParams<float> p, const __grid_constant__ CUtensorMap tm_in,
                           const __grid_constant__ CUtensorMap tm_out) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  pass_begin();
   TwE<float>* s_tw = reinterpret_cast<TwE<float>*>(smem_raw);
   // the tile starts at the first 1024-byte boundary after the twiddles (the swizzle
   // pattern follows the shared-memory address)

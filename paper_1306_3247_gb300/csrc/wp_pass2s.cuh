@@ -257,6 +257,7 @@ constexpr int min_blocks() { return 5; }
 template <int LOGT, int NG, bool SEP>
 __global__ void __launch_bounds__(Geo<LOGT>::THREADS, min_blocks<LOGT>()) k_pass2s_contig(const PassParams<float> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  pass_begin();
   cx<float> v[8];
   contig_load<LOGT>(p.in, blockIdx.x, v);
   contig_body<LOGT, NG, SEP>(p, blockIdx.x, smem_raw, v);
@@ -265,6 +266,7 @@ __global__ void __launch_bounds__(Geo<LOGT>::THREADS, min_blocks<LOGT>()) k_pass
 template <int LOGT, bool KIN>
 __global__ void __launch_bounds__(Geo<LOGT>::THREADS, min_blocks<LOGT>()) k_pass2s_strided(const PassParams<float> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  pass_begin();
   int64_t o, cb;
   strided_origin<LOGT>(p.log_inner, blockIdx.x, o, cb);
   float4 ld[Stage<LOGT>::Q];

@@ -10,9 +10,9 @@ template <int LOGT, int NG>
 void launch_contig_ng(const PassParams<float>& p, unsigned blocks, cudaStream_t st) {
   using G = p2s::Geo<LOGT>;
   if (p.sep)
-    p2s::k_pass2s_contig<LOGT, NG, true><<<blocks, G::THREADS, G::SMEM, st>>>(p);
+    launch_dep(p2s::k_pass2s_contig<LOGT, NG, true>, blocks, G::THREADS, G::SMEM, st, p);
   else
-    p2s::k_pass2s_contig<LOGT, NG, false><<<blocks, G::THREADS, G::SMEM, st>>>(p);
+    launch_dep(p2s::k_pass2s_contig<LOGT, NG, false>, blocks, G::THREADS, G::SMEM, st, p);
 }
 
 template <int LOGT>
@@ -32,9 +32,9 @@ int launch_t(const PassParams<float>& p, cudaStream_t st) {
     else
       launch_contig_ng<LOGT, 0>(q, blocks, st);
   } else if (p.flags & F_KIN) {
-    p2s::k_pass2s_strided<LOGT, true><<<blocks, G::THREADS, G::SMEM, st>>>(p);
+    launch_dep(p2s::k_pass2s_strided<LOGT, true>, blocks, G::THREADS, G::SMEM, st, p);
   } else {
-    p2s::k_pass2s_strided<LOGT, false><<<blocks, G::THREADS, G::SMEM, st>>>(p);
+    launch_dep(p2s::k_pass2s_strided<LOGT, false>, blocks, G::THREADS, G::SMEM, st, p);
   }
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? 0 : (int)e;

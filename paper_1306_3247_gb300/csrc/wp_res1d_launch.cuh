@@ -30,19 +30,28 @@ constexpr int batch_cluster_log() {
   return LOGN <= 12 ? 0 : LOGN - 12;
 }
 
-template <class SH, class K, class... A>
+// DEP: the kernel begins with pass_begin.
+template <class SH, bool DEP, class K, class... A>
 cudaError_t go(K kern, unsigned nlines, cudaStream_t st, A... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(nlines * SH::R);
   cfg.blockDim = dim3(SH::NT + SH::TW);
   cfg.dynamicSmemBytes = SH::SMEM;
   cfg.stream = st;
-  cudaLaunchAttribute at = {};
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = SH::R;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = SH::R > 1 ? 1 : 0;
+  cudaLaunchAttribute at[2] = {};
+  unsigned n = 0;
+  if (DEP) {
+    at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (SH::R > 1) {
+    at[n].id = cudaLaunchAttributeClusterDimension;
+    at[n].val.clusterDim.x = SH::R;
+    at[n].val.clusterDim.y = at[n].val.clusterDim.z = 1;
+    n++;
+  }
+  cfg.attrs = at;
+  cfg.numAttrs = n;
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
@@ -51,7 +60,7 @@ cudaError_t launch_n(const Res1dParams<T>& p, size_t, cudaStream_t st) {
   if constexpr (supported<T, LOGN>()) {
     constexpr int LOGR = cluster_log<LOGN>();
     using SH = line::Shape<T, LOGN, LOGR>;
-    return go<SH>(line::k_line<T, LOGN, LOGR>, 1, st, p);
+    return go<SH, true>(line::k_line<T, LOGN, LOGR>, 1, st, p);
   }
   return cudaErrorInvalidConfiguration;
 }
@@ -61,7 +70,7 @@ cudaError_t launch_batch_n(const Res1dParams<T>* params, int ninst, int64_t nste
   if constexpr (supported<T, LOGN>()) {
     constexpr int LOGR = batch_cluster_log<LOGN>();
     using SH = line::Shape<T, LOGN, LOGR, true>;
-    return go<SH>(line::k_line_batch<T, LOGN, LOGR>, (unsigned)ninst, st, params, nsteps);
+    return go<SH, false>(line::k_line_batch<T, LOGN, LOGR>, (unsigned)ninst, st, params, nsteps);
   }
   return cudaErrorInvalidConfiguration;
 }
