@@ -44,7 +44,10 @@ typedef enum {
 } wp_status;
 
 /* Arithmetic form of the propagation.
- *  WP_C128:       complex128 state, FP64 FFT and phases (the plain FP64 method).
+ *  WP_C128:       complex128 state; transforms and products with the factors in 64-bit
+ *                 fixed point with an exponent per tile (rounding below FP64's) on axes and
+ *                 lines of compile-time length, in FP64 elsewhere; tables and observable
+ *                 sums in FP64. States enter and leave as complex128.
  *  WP_C64:        complex64 state and FFT in FP32; twiddles, phase-argument reductions
  *                 modulo 2 pi and all observable reductions in FP64.
  *  WP_C128_F32X2: complex128 accuracy computed in float-float (pairs of FP32, about 48

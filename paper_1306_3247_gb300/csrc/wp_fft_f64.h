@@ -1,8 +1,8 @@
 // FP64 Stockham butterflies in fused multiply-add form, for the fixed-size transforms of
-// the complex128 path (the Fourier transforms of eq. (ft), Sec. 2.1, and Algorithm 1 of
+// the complex128 passes that apply a grid potential; the others are in fixed point, wp_fx.h (the Fourier transforms of eq. (ft), Sec. 2.1, and Algorithm 1 of
 // arXiv:1306.3247).
 //
-// GB300 runs FP64 at 1/58 of its FP32 rate, so the complex128 passes are bound by the
+// GB300 runs FP64 at 1/58 of its FP32 rate, so an FP64 pass is bound by the
 // FP64 pipe, where an add costs as much as a fused multiply-add. A twiddled butterfly
 // written as complex products followed by sums spends most of its slots on plain adds.
 // Here every twiddle w = exp(i theta) is held in scaled form (the cosine-factor method of

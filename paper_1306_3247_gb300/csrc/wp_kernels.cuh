@@ -1361,11 +1361,11 @@ __global__ void __launch_bounds__(256) k_pass_fixed(const PassParams<T> p) {
   pass_begin();
   pass_body<T, 8, OBS, FixShape<LOGN, CONTIG>, GRID>(p, FixShape<LOGN, CONTIG>(), reinterpret_cast<cx<T>*>(smem_raw));
 }
-// FP64: at most 64 registers, so that four blocks share an SM (the FP64 pipe needs the
-// warps to cover its latency); the passes that also form observable sums or apply a grid
-// potential, at most 80 (three blocks).
-template <int LOGN, bool CONTIG, bool OBS, bool GRID = false>
-__global__ void __launch_bounds__(256, (OBS || GRID) ? 3 : 4) k_pass_fixed_f64(const PassParams<double> p) {
+// FP64: the passes that apply a grid potential (the others are in fixed point), at most 80
+// registers, so that three blocks share an SM (the FP64 pipe needs the warps to cover its
+// latency).
+template <int LOGN, bool CONTIG, bool OBS, bool GRID>
+__global__ void __launch_bounds__(256, 3) k_pass_fixed_f64(const PassParams<double> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   pass_begin();
   pass_body<double, 8, OBS, FixShape<LOGN, CONTIG>, GRID>(p, FixShape<LOGN, CONTIG>(),

@@ -1,9 +1,9 @@
 // Arithmetic-rate probe: the FP64 and FP32 fused multiply-add throughput of the device.
 //
-// The paper has no counterpart of this entry point. It measures the rate that bounds the
-// native FP64 form of the split step on GB300 (whose FP64 pipe, not HBM, sets the pace of
-// a complex128 pass), so that a roofline fraction of that form can be stated against a
-// rate measured on the same device in the same run.
+// The paper has no counterpart of this entry point. It measures the rates
+// of the pipes that carry the split step on GB300 (FP64: tables, sums and grid-potential
+// passes of the complex128 form; FP32: the other forms), so that the work of a pass can be
+// stated against a rate measured on the same device in the same run.
 //
 // Method: every thread runs 8 independent FMA chains x <- x b + a (b just below 1, so the
 // values stay bounded), enough warps per SM to cover the pipe latency (8 blocks of 256
