@@ -46,7 +46,8 @@ from paper_1306_3247_gb300 import workloads as W  # noqa: E402
 METRIC = "grid-point·steps/s (256³ c128 plain vs batched c64) + served p50/p99 ms"
 UNIT = "grid-point·steps/s"
 # DRAM bytes (read + write) per launch of each pass class on the 256^3 workload, from one
-# ncu capture of the current kernels (dram__bytes_read.sum + dram__bytes_write.sum). Valid
+# ncu capture (dram__bytes_read.sum + dram__bytes_write.sum; of the FP64 passes for c128, which
+# swept the same state once a pass as the fixed-point ones do). Valid
 # for grid 256 only; any other grid reports null.
 TRAFFIC_256 = {
     "c128": {"pass_contig": 480336128, "pass_strided": 472172288, "pass_kinetic": 477476096},

@@ -1,19 +1,19 @@
 // Passes of the complex128 form in 64-bit fixed point (wp_fx.h): a tile is held as integers
-// with one exponent through the transforms and factors of the pass. Tiles, stage plan and
-// thread mapping are those of the fixed-shape kernels of wp_kernels.cuh (2048 points, 256
+// with one exponent through the transforms and factors of the pass. Tiles and stage plan are
+// those of the fixed-shape kernels of wp_kernels.cuh (2048 points, 256
 // threads, n = 32..2048, the lengths whose stages unroll); those that form observable sums
 // add them up in FP64 from the results; passes that apply a grid potential stay in FP64.
 //
-// Bound by the integer pipe (64 lanes per clock; ncu on 256^3: 61 % busy over the launch,
-// FP64 before 92 %) and by instruction issue (62 %). Measured on the 256^3 barrier, CUDA
-// events in the step, FP64 before and fixed point now: FFT-only pass 617 -> 162 us, kinetic
-// pass 1411 -> 333 us, potential pass 1118 -> 352 us.
+// Bound by the integer pipe (64 lanes per clock; ncu on 256^3: 63-69 % busy, FP64 before
+// 92 %) and by instruction issue. Measured on the 256^3 barrier, CUDA events in the step, FP64
+// before, fixed point with the whole tile in shared memory, and these: FFT-only pass 617, 162,
+// 159 us; kinetic pass 1411, 333, 322; potential pass 1118, 352, 290. The FP64 pipe bounds the
+// sums of a record (86 % busy in the position sums, 489 us).
 //
 // In memory a state is complex128 at the ends of a chunk of steps and in fixed point between
 // its passes (F_IN_FX, F_OUT_FX): the conversions between doubles and integers are about
 // 130 instructions per point and pass, those of the stored fixed-point form about 40 (FFT-only
 // pass 187 -> 162 us under ncu).
-//
 #pragma once
 
 #include "wp_fx.h"
