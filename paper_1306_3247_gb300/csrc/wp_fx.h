@@ -145,8 +145,9 @@ WP_HD FxSchedule fx_schedule(int32_t bM, int32_t bS) {
   r.total = B[ns] - 62;
   return r;
 }
-// Lines of 2^11 points and more take their bound anew after 64 points (span 2^6): the line
-// sum alone is far above the values that a long line of many comparable points forms.
+// Resident lines of 2^11 points and more take their bound anew after 64 points (span 2^6): the
+// line sum alone is far above the values that a long line of many comparable points forms.
+// Passes take the bound of their inputs through to the end.
 constexpr int kFxMidLog = 6;
 WP_HD constexpr bool fx_mid(int logn) { return logn >= 11; }
 
@@ -191,12 +192,28 @@ WP_HD void fx_dft(cx<int64_t>* v) {
   }
 }
 
-// |x| / 2^43 rounded up, of a double with high word hi and its leading one at bit 62 - s.
+// Units of the 32-bit sums of |re| + |im| of a line, 2^UNIT. A part is below 2^63 and its
+// magnitude rounded up at most 2^(63 - UNIT) units, so a line of n points sums to at most
+// n 2^(64 - UNIT): below 2^32 for the 2048 points of a pass in units of 2^44 (in units of 2^43
+// a flat line just below a power of two is 2^32 and its sum 0), and for the 8192 of a resident
+// line in units of 2^46.
+constexpr int kFxPassSum = 44, kFxLineSum = 46;
+
+// |x| / 2^UNIT rounded up, of a double with high word hi and its leading one at bit 62 - s.
+template <int UNIT = 43>
 WP_HD uint32_t fx_mag(uint32_t hi, uint32_t s) {
-  return fx_shr64(((hi & 0x000fffffu) | 0x00100000u) >> 1, 0u, s) + 1u;
+  return fx_shr64(((hi & 0x000fffffu) | 0x00100000u) >> (UNIT - 42), 0u, s) + 1u;
 }
-// Bits of a line sum in units of 2^43.
-WP_HD int32_t fx_sum_bits(uint32_t L) { return 75 - fx_clz(L); }
+// |x| / 2^UNIT rounded up, of an integer x with high word a of its magnitude rounded down.
+template <int UNIT>
+WP_HD uint32_t fx_mag_int(uint32_t a) {
+  return (a >> (UNIT - 32)) + 1u;
+}
+// Bits of a line sum in units of 2^UNIT.
+template <int UNIT = 43>
+WP_HD int32_t fx_sum_bits(uint32_t L) {
+  return 32 + UNIT - fx_clz(L);
+}
 
 // The double with words (hi, lo), its leading one moved to bit 62 - s. The last bit is set,
 // which makes the error of the dropped bits symmetric (a plain floor would leave half a unit

@@ -250,10 +250,10 @@ __device__ __forceinline__ bool pass(const PassParams<double>& p, void* smem, in
       const uint32_t d = m - fx_code(wlo(v[k].re), wlo(v[k].im));
       const uint32_t ar = fx_shr64(absh(whi(v[k].re)), 0u, d), ai = fx_shr64(absh(whi(v[k].im)), 0u, d);
       any |= ar | ai;
-      L += (ar >> 11) + (ai >> 11) + 2u;
+      L += fx_mag_int<kFxPassSum>(ar) + fx_mag_int<kFxPassSum>(ai);
     }
     const uint32_t Lm = ti.sum(L, any, red[0], redm[1]);
-    sc = fx_schedule<LOGN>(65 - __clz((int)any), fx_sum_bits(Lm));
+    sc = fx_schedule<LOGN>(65 - __clz((int)any), fx_sum_bits<kFxPassSum>(Lm));
     ex = (int32_t)m - kFxBias + sc.first;
     const uint32_t right = sc.first > 0 ? (uint32_t)sc.first : 0u, left = sc.first < 0 ? (uint32_t)-sc.first : 0u;
 #pragma unroll
@@ -283,11 +283,11 @@ __device__ __forceinline__ bool pass(const PassParams<double>& p, void* smem, in
     const uint32_t E = m >> 20;
 #pragma unroll
     for (int k = 0; k < 8; k++) {
-      L += fx_mag(whi(v[k].re), E - ((whi(v[k].re) >> 20) & 0x7ffu));
-      L += fx_mag(whi(v[k].im), E - ((whi(v[k].im) >> 20) & 0x7ffu));
+      L += fx_mag<kFxPassSum>(whi(v[k].re), E - ((whi(v[k].re) >> 20) & 0x7ffu));
+      L += fx_mag<kFxPassSum>(whi(v[k].im), E - ((whi(v[k].im) >> 20) & 0x7ffu));
     }
     uint32_t any = 0;
-    sc = fx_schedule<LOGN>(64, fx_sum_bits(ti.sum(L, any, red[0], redm[1])));
+    sc = fx_schedule<LOGN>(64, fx_sum_bits<kFxPassSum>(ti.sum(L, any, red[0], redm[1])));
     const uint32_t E2 = E + (uint32_t)sc.first;
     ex = (int32_t)E2 + off;
 #pragma unroll
@@ -351,12 +351,12 @@ __device__ __forceinline__ bool pass(const PassParams<double>& p, void* smem, in
     for (int k = 0; k < 8; k++) {
       const uint32_t ar = absh(x[k].re), ai = absh(x[k].im);
       any |= ar | ai;
-      L += (ar >> 11) + (ai >> 11) + 2u;
+      L += fx_mag_int<kFxPassSum>(ar) + fx_mag_int<kFxPassSum>(ai);
     }
     if (t0 && t1) {
       // the transform before has changed the bounds: a new scale
       const uint32_t Lm = ti.sum(L, any, red[1], redm[2]);
-      sc = fx_schedule<LOGN>(65 - __clz((int)any), fx_sum_bits(Lm));
+      sc = fx_schedule<LOGN>(65 - __clz((int)any), fx_sum_bits<kFxPassSum>(Lm));
       ex += sc.first;
 #pragma unroll
       for (int k = 0; k < 8; k++) x[k] = mk(shift_jam(x[k].re, sc.first), shift_jam(x[k].im, sc.first));

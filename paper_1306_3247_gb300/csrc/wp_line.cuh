@@ -213,10 +213,10 @@ struct Line {
     for (int k = 0; k < P; k++) {
       const uint32_t ar = fxp::absh(x[k].re), ai = fxp::absh(x[k].im);
       any |= ar | ai;
-      L += (ar >> 14) + (ai >> 14) + 2u;
+      L += fx_mag_int<kFxLineSum>(ar) + fx_mag_int<kFxLineSum>(ai);
     }
     reduce(any, L);
-    bS = 78 - __clz((int)L);  // units of 2^46
+    bS = fx_sum_bits<kFxLineSum>(L);
     constexpr int LS1 = fx_mid(LOGN) ? kFxMidLog : LOGN;
     const FxSchedule sc = fx_schedule<LOGN, 0, LS1>(65 - __clz((int)any), bS);
     ex += sc.total;
