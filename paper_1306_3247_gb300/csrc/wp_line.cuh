@@ -635,6 +635,30 @@ __device__ __forceinline__ void body(const Res1dParams<T>& p, unsigned char* sme
       return v;
     }
   };
+  const bool obs = !BATCH && p.obs;
+  [[maybe_unused]] const DevPot& pot = *p.pot;
+  [[maybe_unused]] const double tm0 = p.g.t0 + (double)(s0 + m) * dt;
+  // The potential of a record, point by point: its linear terms from the sums of x |psi|^2 and
+  // |psi|^2 would cancel on a box far from the origin. The general terms follow below.
+  [[maybe_unused]] double W[P];
+  if (obs) {
+    ln.bar();
+    if (t < pot.nterms) fco[0][t] = term_coef(pot.term[t], tm0);
+    ln.bar();
+#pragma unroll
+    for (int k = 0; k < P; k++) W[k] = p.Vs[ln.point(k)];
+    for (int e = 0; e < pot.nterms; e++) {
+      if (!((p.plane_mask >> e) & 1u)) continue;
+      const wp_pot_term& tm = pot.term[e];
+      const bool lin = tm.shape == WP_SHAPE_LINEAR;
+      const double f = lin ? fco[0][e] * tm.a[0] : fco[0][e], ctr = tm.c0[0] + tm.v[0] * tm0;
+#pragma unroll
+      for (int k = 0; k < P; k++) {
+        const double xi = p.g.xmin[0] + (double)ln.point(k) * p.g.dx[0];
+        W[k] = lin ? fma(f, xi - ctr, W[k]) : W[k] + f;
+      }
+    }
+  }
   double acc[NQ];
 #pragma unroll
   for (int q = 0; q < NQ; q++) acc[q] = 0.0;
@@ -643,14 +667,13 @@ __device__ __forceinline__ void body(const Res1dParams<T>& p, unsigned char* sme
     const int i = ln.point(k);
     const cx<T> v = value(x[k]);
     if (m > 0) p.psi[i] = v;
-    if (!BATCH && p.obs) {
-      // V = V_s + beta x - gamma + general terms: the plane part from the moments below
+    if (obs) {
       const double re = to_f64(v.re), im = to_f64(v.im);
       const double rho = fma(re, re, im * im), xi = p.g.xmin[0] + (double)i * p.g.dx[0], xr = xi * rho;
       acc[Q_RHO] += rho;
       acc[Q_X] += xr;
       acc[Q_XX] += xi * xr;
-      acc[Q_V] += p.Vs[i] * rho;
+      acc[Q_V] += W[k] * rho;
       if (p.autocorr) {
         const cx<T> z = p.psi0[i];
         const double zr = to_f64(z.re), zi = to_f64(z.im);
@@ -659,12 +682,7 @@ __device__ __forceinline__ void body(const Res1dParams<T>& p, unsigned char* sme
       }
     }
   }
-  if (!BATCH && p.obs) {
-    const DevPot& pot = *p.pot;
-    const double tm0 = p.g.t0 + (double)(s0 + m) * dt;
-    ln.bar();
-    if (t < pot.nterms) fco[0][t] = term_coef(pot.term[t], tm0);
-    ln.bar();
+  if (obs) {
     if (p.gen_mask) {
 #pragma unroll 1
       for (int k = 0; k < P; k++) {
@@ -699,20 +717,7 @@ __device__ __forceinline__ void body(const Res1dParams<T>& p, unsigned char* sme
       acc[Q_K2] += kk * kr;
     }
     total(ln, acc, (1u << Q_RHOK) | (1u << Q_K) | (1u << Q_K2), redd, part[1], 1, qm);
-    if (t < 32 && c == 0u) {
-      if (t == 0) {
-        for (int e = 0; e < pot.nterms; e++) {
-          if (!((p.plane_mask >> e) & 1u)) continue;
-          const wp_pot_term& tm = pot.term[e];
-          if (tm.shape == WP_SHAPE_LINEAR)
-            qp[Q_V] += fco[0][e] * tm.a[0] * (qp[Q_X] - (tm.c0[0] + tm.v[0] * tm0) * qp[Q_RHO]);
-          else
-            qp[Q_V] += fco[0][e] * qp[Q_RHO];
-        }
-      }
-      __syncwarp();
-      publish_obs(qp, qm, p.g, p.autocorr, tm0, s0 + m, t, p.ctrl, p.obs_out, p.obs_cap);
-    }
+    if (t < 32 && c == 0u) publish_obs(qp, qm, p.g, p.autocorr, tm0, s0 + m, t, p.ctrl, p.obs_out, p.obs_cap);
   }
   if (t == 0 && c == 0u) p.ctrl->step = s0 + m;
   if constexpr (SH::TW > 0) __syncthreads();
