@@ -38,7 +38,8 @@ typedef enum {
   WP_EUNSUPPORTED = 2,  /* size not a power of two, ndim outside 1..3, too large a line */
   WP_ENOMEM = 3,        /* device allocation failed */
   WP_ENONFINITE = 4,    /* the norm became NaN or infinite */
-  WP_ETIMEOUT = 5,      /* a bounded device wait gave up */
+  WP_ETIMEOUT = 5,      /* a bounded device wait gave up: the state is not valid; returned by the next
+                           call on the handle that synchronises and returns host data, once */
   WP_ECUDA = 6,         /* any other CUDA error; see wp_last_error */
   WP_EBUSY = 7          /* the handle is in use (e.g. a batch slot is occupied) */
 } wp_status;

@@ -152,7 +152,7 @@ struct Ctrl {
   double t_tab;                  // time of the current potential tables
   double gphase[WP_MAX_GAUSS];   // f_g(t) tau / hbar for the Gaussian terms
   double gcoef[WP_MAX_GAUSS];    // f_g(t)
-  int32_t err;                   // first error raised by a kernel (0 = none)
+  int32_t err;                   // worst error raised by a kernel (0 = none); WP_ETIMEOUT stays until read
   uint32_t prep_done;            // blocks of the current k_prep launch that have finished
 };
 

@@ -150,12 +150,12 @@ struct Line {
   uint32_t (*red)[32];   // [2][32]: block reductions
   uint32_t (*cred)[2][8];  // [2]: the cluster's
   uint64_t* mb;          // mbarriers: [0..1] buffers, [2..3] cluster reductions, [4..5] records
-  int32_t* err;
+  Ctrl* ctrl;
   int32_t ex;            // fixed point: an integer x stands for x 2^(ex - 1085)
   int t;
   uint32_t c;            // rank in the cluster
   uint32_t nfft, nred;   // exchanges so far: buffer n & 1, phase parity (n >> 1) & 1
-  bool lost;             // a wait has run out: the rest of the chunk no longer waits
+  bool lost;             // a wait has run out: the rest of the chunk no longer waits, and the thread's points are lost
 
   __device__ __forceinline__ int point(int k) const { return (int)c + R * (t + k * NT); }
   // Barrier of the block's transforming threads.
@@ -167,7 +167,7 @@ struct Line {
     for (int k = 0; k < (1 << 20); k++)
       if (try_wait(pair + (n & 1u), (n >> 1) & 1u)) return;
     lost = true;
-    atomicCAS(err, 0, (int32_t)WP_ETIMEOUT);
+    raise_error(ctrl, WP_ETIMEOUT);
   }
 
   // (union, sum) of the line's (any, L), in every thread.
@@ -470,7 +470,7 @@ __device__ __forceinline__ void body(const Res1dParams<T>& p, unsigned char* sme
       return;
     }
   }
-  LN ln{s, red, cred, mb, &p.ctrl->err, 0, t, c, 0u, 0u, false};
+  LN ln{s, red, cred, mb, p.ctrl, 0, t, c, 0u, 0u, false};
   V x[P];
   bool zero = false;
   int bad = 0;
@@ -665,7 +665,8 @@ __device__ __forceinline__ void body(const Res1dParams<T>& p, unsigned char* sme
 #pragma unroll
   for (int k = 0; k < P; k++) {
     const int i = ln.point(k);
-    const cx<T> v = value(x[k]);
+    cx<T> v = value(x[k]);
+    if (R > 1 && ln.lost) v = mk(T(qnan), T(qnan));  // never taken for a result
     if (m > 0) p.psi[i] = v;
     if (obs) {
       const double re = to_f64(v.re), im = to_f64(v.im);
