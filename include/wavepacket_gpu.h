@@ -46,7 +46,7 @@ typedef enum {
 
 /* Arithmetic form of the propagation.
  *  WP_C128:       complex128 state; transforms and products with the factors in 64-bit
- *                 fixed point with an exponent per tile (rounding below FP64's) on axes and
+ *                 fixed point with an exponent per line (rounding below FP64's) on axes and
  *                 lines of compile-time length, in FP64 elsewhere; tables and observable
  *                 sums in FP64. States enter and leave as complex128.
  *  WP_C64:        complex64 state and FFT in FP32; twiddles, phase-argument reductions

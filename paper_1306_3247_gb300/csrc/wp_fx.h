@@ -6,11 +6,11 @@
 // integer ones per clock, so a complex128 pass written in FP64 is bound by that pipe: a
 // 256-point transform is about 20 FP64 instructions per point, 1500 issue slots' worth.
 // Between the load and the store of a pass a line is therefore held as 64-bit integers with
-// one common exponent per tile. A sum is exact and costs about 3.4 issue slots, a product
+// one common exponent per line. A sum is exact and costs about 3.4 issue slots, a product
 // with a unit factor about 60 (measured on GB300, 32-bit multiplies and high words).
 //
-// Accuracy. With M the largest |x| of a tile and S the largest sum(|re| + |im|) of its
-// lines, every value a transform forms from q of a line's points is at most min(q M, S). The
+// Accuracy. With M the largest |x| of a line and S its sum of |re| + |im|,
+// every value a transform forms from q of its points is at most min(q M, S). The
 // integers are scaled stage by stage so that this bound stays below 2^62 (fx_schedule):
 // nothing overflows, and no bits are kept back for growth that a line cannot have. The few
 // roundings (one when a double becomes an integer, one per product) are a small number of
@@ -259,15 +259,16 @@ WP_HD void fx_to_double(int64_t v, int32_t e, uint32_t& hi, uint32_t& lo) {
 // point below the range, kFxNan one that is not finite.
 constexpr int32_t kFxBias = 1200, kFxNan = 4095;
 WP_HD uint32_t fx_code(uint32_t re_lo, uint32_t im_lo) { return ((re_lo & 63u) << 6) | (im_lo & 63u); }
-// v >> s with the six code bits replaced by their middle and the last bit set.
-WP_HD int64_t fx_align(uint32_t lo, int32_t hi, uint32_t s) {
+// v >> s with the six code bits replaced by their middle and the last bit set (jam = 0: left
+// as it is, so that a zero far below the line's largest stays zero).
+WP_HD int64_t fx_align(uint32_t lo, int32_t hi, uint32_t s, uint32_t jam = 1u) {
   const bool far = s >= 32u;
   uint32_t l = (lo & ~63u) | 32u;
   const int32_t sg = hi >> 31;
   l = far ? (uint32_t)hi : l;
   const int32_t h = far ? sg : hi;
   s = far ? s - 32u : s;
-  const uint32_t r = fx_shr64(l, (uint32_t)h, s) | 1u;
+  const uint32_t r = fx_shr64(l, (uint32_t)h, s) | jam;
   return (int64_t)(((uint64_t)(uint32_t)(h >> (s > 31u ? 31u : s)) << 32) | r);
 }
 

@@ -1,5 +1,5 @@
-// Passes of the complex128 form in 64-bit fixed point (wp_fx.h): a tile is held as integers
-// with one exponent through the transforms and factors of the pass. Tiles and stage plan are
+// Passes of the complex128 form in 64-bit fixed point (wp_fx.h): each line of a tile is held as
+// integers with one exponent through the transforms and factors of the pass. Tiles and stage plan are
 // those of the fixed-shape kernels of wp_kernels.cuh (2048 points, 256
 // threads, n = 32..2048, the lengths whose stages unroll); those that form observable sums
 // add them up in FP64 from the results; passes that apply a grid potential stay in FP64.
@@ -29,6 +29,24 @@ __device__ __forceinline__ uint32_t wlo(double x) { return (uint32_t)__double2lo
 // The high word of |v|, rounded down, from that of v.
 __device__ __forceinline__ uint32_t absh(uint32_t h) { return h ^ (uint32_t)((int32_t)h >> 31); }
 __device__ __forceinline__ uint32_t absh(int64_t v) { return absh((uint32_t)(v >> 32)); }
+
+struct Max {
+  static __device__ __forceinline__ uint32_t two(uint32_t a, uint32_t b) { return max(a, b); }
+  static __device__ __forceinline__ uint32_t warp(uint32_t v) { return __reduce_max_sync(0xffffffffu, v); }
+};
+struct Or {
+  static __device__ __forceinline__ uint32_t two(uint32_t a, uint32_t b) { return a | b; }
+  static __device__ __forceinline__ uint32_t warp(uint32_t v) { return __reduce_or_sync(0xffffffffu, v); }
+};
+struct Add {
+  static __device__ __forceinline__ uint32_t two(uint32_t a, uint32_t b) { return a + b; }
+  static __device__ __forceinline__ uint32_t warp(uint32_t v) { return __reduce_add_sync(0xffffffffu, v); }
+};
+
+// The shifts of a schedule's stages, two bits each.
+__device__ __forceinline__ uint32_t packed(const FxSchedule& sc) {
+  return sc.at[0] | (sc.at[1] << 2) | (sc.at[2] << 4) | (sc.at[3] << 6);
+}
 
 // A tile's lines in registers and shared memory: thread t of a line's n/8 threads holds the
 // points t + k n/8, which are the inputs of its butterfly in the first Stockham stage and its
@@ -75,48 +93,69 @@ struct Tile {
       __syncthreads();
   }
 
-  // The largest line sum of the tile (L: the thread's part of its line's) and the union of
-  // the threads' `any`. red, redm: 256 and 8 words, not used by anything else between the
-  // barriers before and after the call.
-  __device__ __forceinline__ uint32_t sum(uint32_t L, uint32_t& any, uint32_t* red, uint32_t* redm) const {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    any = __reduce_or_sync(0xffffffffu, any);
-    if (lane == 0) redm[warp] = any;
-    uint32_t r = 0;
-    if constexpr (CONTIG) {
+  // Reductions over the threads of a line. Where they are lanes of one warp (contiguous axes
+  // up to 256 points) it is done in it; else the warps' parts cross shared memory (red: 256
+  // words, not used by anything else between the barriers before and after the call).
+  static constexpr bool IN_WARP = CONTIG && TL <= 32;
+  template <class Op>
+  static __device__ __forceinline__ uint32_t warp_part(uint32_t v) {
+    if constexpr (CONTIG && TL >= 32) {
+      v = Op::warp(v);
+    } else {
 #pragma unroll
-      for (int o = 1; o < (TL < 32 ? TL : 32); o <<= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
-      if constexpr (TL < 32) L = __reduce_max_sync(0xffffffffu, L);
-      if (lane == 0) red[warp] = L;
-      __syncthreads();
+      for (int o = CONTIG ? 1 : C; o < (CONTIG ? TL : 32); o <<= 1) v = Op::two(v, __shfl_xor_sync(0xffffffffu, v, o));
+    }
+    return v;
+  }
+  static __device__ __forceinline__ void put(uint32_t v, uint32_t* red) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if constexpr (CONTIG) {
+      if (lane == 0) red[warp] = v;
+    } else {
+      if (lane < C) red[warp * 32 + lane] = v;
+    }
+  }
+  template <class Op>
+  static __device__ __forceinline__ uint32_t get(const uint32_t* red) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t v = 0;
+    if constexpr (CONTIG) {
       constexpr int WL = TL < 32 ? 1 : TL / 32;  // warps of a line
 #pragma unroll
-      for (int w = 0; w < 8; w += WL) {
-        uint32_t u = 0;
-#pragma unroll
-        for (int k = 0; k < WL; k++) u += red[w + k];
-        r = max(r, u);
-      }
+      for (int k = 0; k < WL; k++) v = Op::two(v, red[(warp & ~(WL - 1)) + k]);
     } else {
-      constexpr int CW = C < 32 ? C : 32;  // lines a warp meets; of 64 lines odd and even warps meet one half each
+      // every warp meets every column; of 64 columns odd and even warps one half each
 #pragma unroll
-      for (int o = C; o < 32; o <<= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
-      if (lane < CW) red[warp * CW + lane] = L;
-      __syncthreads();
-      uint32_t u[2] = {0, 0};
-#pragma unroll
-      for (int w = 0; w < 8; w++) u[C > 32 ? w & 1 : 0] += red[w * CW + (lane & (CW - 1))];
-      r = __reduce_max_sync(0xffffffffu, max(u[0], u[1]));
+      for (int k = 0; k < 8; k += C > 32 ? 2 : 1)
+        v = Op::two(v, red[(k + (C > 32 ? warp & 1 : 0)) * 32 + (lane & (C - 1))]);
     }
-#pragma unroll
-    for (int w = 0; w < 8; w++) any |= redm[w];
-    return r;
+    return v;
+  }
+  static __device__ __forceinline__ void line_max(uint32_t& m, uint32_t* red) {
+    m = warp_part<Max>(m);
+    if constexpr (!IN_WARP) {
+      put(m, red);
+      __syncthreads();
+      m = get<Max>(red);
+    }
+  }
+  // (union, sum) of the line's (any, L)
+  static __device__ __forceinline__ void line_bounds(uint32_t& any, uint32_t& L, uint32_t* ra, uint32_t* rl) {
+    any = warp_part<Or>(any);
+    L = warp_part<Add>(L);
+    if constexpr (!IN_WARP) {
+      put(any, ra);
+      put(L, rl);
+      __syncthreads();
+      any = get<Or>(ra);
+      L = get<Add>(rl);
+    }
   }
 
-  // The forward transform of the tile's lines, with the scaling of sc. The inverse one is the
+  // The forward transform of the line, with the shifts of its schedule (packed). The inverse one is the
   // same on points with real and imaginary parts exchanged, before and after.
   template <int LOGNS = 0, int S = 0>
-  __device__ __forceinline__ void fft(cx<int64_t> (&x)[8], const FxRec* __restrict__ tw, const FxSchedule& sc) const {
+  __device__ __forceinline__ void fft(cx<int64_t> (&x)[8], const FxRec* __restrict__ tw, uint32_t shifts) const {
     constexpr int LR = wp_stage_radix_log(LOGN, LOGNS), R = 1 << LR, B = 8 / R, NS = 1 << LOGNS;
     if constexpr (LOGNS > 0) {
 #pragma unroll
@@ -128,7 +167,7 @@ struct Tile {
 #pragma unroll
       for (int r = 0; r < R; r++) v[r] = x[b + B * r];
       if constexpr (LOGNS > 0) {
-        const uint32_t sh = sc.at[S];
+        const uint32_t sh = (shifts >> (2 * S)) & 3u;
         const FxRec* e = tw + wp_stage_tw_offset(LOGN, LOGNS) + ((t + b * TL) & (NS - 1));
         v[0] = mk(v[0].re >> (2u - sh), v[0].im >> (2u - sh));
 #pragma unroll
@@ -148,7 +187,7 @@ struct Tile {
         for (int r = 0; r < R; r++) at(d0 + (r << LOGNS)) = x[b + B * r];
       }
       sync();
-      fft<LOGNS + LR, S + 1>(x, tw, sc);
+      fft<LOGNS + LR, S + 1>(x, tw, shifts);
     }
   }
 };
@@ -196,55 +235,33 @@ __device__ __noinline__ int gauss_points(TI ti, double a0, double a1, const doub
   return bad;
 }
 
-// v: the thread's points, loaded by the caller. OBS: v returns the pass's results as doubles
-// for the sums, unless the tile is empty or not finite: then its row of the sums is written
-// here and the result is false.
+// v: the thread's points, loaded by the caller. OBS: v returns the pass's results as doubles,
+// for the sums.
 template <int LOGN, bool CONTIG, bool OBS>
-__device__ __forceinline__ bool pass(const PassParams<double>& p, void* smem, int64_t tile, cx<double> (&v)[8]) {
+__device__ __forceinline__ void pass(const PassParams<double>& p, void* smem, int64_t tile, cx<double> (&v)[8]) {
   using TI = Tile<LOGN, CONTIG>;
   constexpr int TL = TI::TL;
-  __shared__ uint32_t red[2][256];
-  __shared__ uint32_t redm[3][8];
+  __shared__ uint32_t red[TI::IN_WARP ? 1 : 4][TI::IN_WARP ? 1 : 256];
+  constexpr int R1 = TI::IN_WARP ? 0 : 1, R2 = 2 * R1, R3 = 3 * R1;
   const TI ti(smem);
-  const int tid = threadIdx.x;
   const uint32_t f = p.flags;
   const FxRec* tw = reinterpret_cast<const FxRec*>(p.Wln);
-  int64_t step;
-  cx<double>* dst = p.out + ti.base(p.log_inner, tile, step);
   const bool in_fx = (f & F_IN_FX) && p.fx_state, out_fx = (f & F_OUT_FX) && p.fx_state;
 
-  // Load: the tile's exponent (the largest leading bit), its bounds M and S, the integers.
-  // An integer x of the tile stands for x 2^(ex - 1085).
-  auto tile_max = [&](uint32_t m) {
-    m = __reduce_max_sync(0xffffffffu, m);
-    if ((tid & 31) == 0) redm[0][tid >> 5] = m;
-    __syncthreads();
-#pragma unroll
-    for (int w = 0; w < 8; w++) m = max(m, redm[0][w]);
-    return m;
-  };
-  // a tile that is all zero stays so; a value that is not finite spoils its tile
-  auto fill = [&](bool finite) {
-    const double z = finite ? 0.0 : (out_fx ? __longlong_as_double(63) : __longlong_as_double(0x7ff8000000000000ll));
-#pragma unroll
-    for (int k = 0; k < 8; k++)
-      if (!OBS || !(f & F_NO_STORE)) dst[k * step] = mk(z, z);
-    if (OBS && tid < NQ) p.partials[tile * NQ + tid] = z;
-    return false;
-  };
-  FxSchedule sc;
+  // Load: the line's exponent (the largest leading bit), its bounds M and S, the integers.
+  // An integer x of the line stands for x 2^(ex - 1085). A line that is all zero stays so; a
+  // value that is not finite spoils its line.
   int32_t ex;
-  uint32_t L = 0;
+  uint32_t shifts, L = 0, any = 0, m = 0;
+  enum { FINITE, ZERO, SPOIL } kind = FINITE;
   const bool ph = CONTIG && (f & F_PHASE), kin = !CONTIG && (f & F_KIN);
   bool swap = (f & F_IFFT) != 0;  // whether the points have their parts exchanged
   cx<int64_t> x[8];
   if (in_fx) {
-    uint32_t m = 0;
 #pragma unroll
     for (int k = 0; k < 8; k++) m = max(m, fx_code(wlo(v[k].re), wlo(v[k].im)));
-    m = tile_max(m);
-    if (m == 0u || m == (uint32_t)kFxNan) return fill(m == 0u);
-    uint32_t any = 0;
+    ti.line_max(m, red[0]);
+    kind = m == 0u ? ZERO : m == (uint32_t)kFxNan ? SPOIL : FINITE;
 #pragma unroll
     for (int k = 0; k < 8; k++) {
       const uint32_t d = m - fx_code(wlo(v[k].re), wlo(v[k].im));
@@ -252,44 +269,43 @@ __device__ __forceinline__ bool pass(const PassParams<double>& p, void* smem, in
       any |= ar | ai;
       L += fx_mag_int<kFxPassSum>(ar) + fx_mag_int<kFxPassSum>(ai);
     }
-    const uint32_t Lm = ti.sum(L, any, red[0], redm[1]);
-    sc = fx_schedule<LOGN>(65 - __clz((int)any), fx_sum_bits<kFxPassSum>(Lm));
-    ex = (int32_t)m - kFxBias + sc.first;
+    ti.line_bounds(any, L, red[R1], red[R2]);
+    const FxSchedule sc = fx_schedule<LOGN>(65 - __clz((int)any), fx_sum_bits<kFxPassSum>(L));
+    ex = (int32_t)m - kFxBias + sc.total;  // that of the transform's results
+    shifts = packed(sc);
     const uint32_t right = sc.first > 0 ? (uint32_t)sc.first : 0u, left = sc.first < 0 ? (uint32_t)-sc.first : 0u;
 #pragma unroll
     for (int k = 0; k < 8; k++) {
-      const uint32_t rl = wlo(v[k].re), il = wlo(v[k].im), d = m - fx_code(rl, il) + right;
-      x[k] = mk((int64_t)((uint64_t)fx_align(rl, (int32_t)whi(v[k].re), d) << left),
-                (int64_t)((uint64_t)fx_align(il, (int32_t)whi(v[k].im), d) << left));
+      const uint32_t rl = wlo(v[k].re), il = wlo(v[k].im), c = fx_code(rl, il), d = m - c + right, jam = min(c, 1u);
+      x[k] = mk((int64_t)((uint64_t)fx_align(rl, (int32_t)whi(v[k].re), d, jam) << left),
+                (int64_t)((uint64_t)fx_align(il, (int32_t)whi(v[k].im), d, jam) << left));
     }
   } else {
-    auto top = [&] {
-      uint32_t m = 0;
 #pragma unroll
-      for (int k = 0; k < 8; k++) m = max(m, max(whi(v[k].re) & 0x7fffffffu, whi(v[k].im) & 0x7fffffffu));
-      return tile_max(m);
-    };
-    uint32_t m = top();
-    int32_t off = 0;  // the integers hold the tile times 2^-off
-    if (m < (70u << 20)) {
-      // all below 2^-953: lift the tile off the denormals
-      __syncthreads();
-      off = -900;
+    for (int k = 0; k < 8; k++) m = max(m, max(whi(v[k].re) & 0x7fffffffu, whi(v[k].im) & 0x7fffffffu));
+    ti.line_max(m, red[0]);
+    // all below 2^-953: lifted off the denormals, whose exponent field stands for 1
+    const bool low = m < (70u << 20);
+    uint32_t E = m >> 20;
+    if (low) {
+      E = max(E, 1u) + 900u;
 #pragma unroll
-      for (int k = 0; k < 8; k++) v[k] = mk(v[k].re * 0x1p900, v[k].im * 0x1p900);
-      m = top();
+      for (int k = 0; k < 8; k++) {
+        any |= wlo(v[k].re) | wlo(v[k].im);
+        v[k] = mk(v[k].re * 0x1p900, v[k].im * 0x1p900);
+      }
     }
-    if (m == 0u || m >= 0x7ff00000u) return fill(m == 0u);
-    const uint32_t E = m >> 20;
 #pragma unroll
     for (int k = 0; k < 8; k++) {
       L += fx_mag<kFxPassSum>(whi(v[k].re), E - ((whi(v[k].re) >> 20) & 0x7ffu));
       L += fx_mag<kFxPassSum>(whi(v[k].im), E - ((whi(v[k].im) >> 20) & 0x7ffu));
     }
-    uint32_t any = 0;
-    sc = fx_schedule<LOGN>(64, fx_sum_bits<kFxPassSum>(ti.sum(L, any, red[0], redm[1])));
+    ti.line_bounds(any, L, red[R1], red[R2]);
+    kind = (m | any) == 0u ? ZERO : m >= 0x7ff00000u ? SPOIL : FINITE;
+    const FxSchedule sc = fx_schedule<LOGN>(64, fx_sum_bits<kFxPassSum>(L));
     const uint32_t E2 = E + (uint32_t)sc.first;
-    ex = (int32_t)E2 + off;
+    ex = (int32_t)E + sc.total - (low ? 900 : 0);
+    shifts = packed(sc);
 #pragma unroll
     for (int k = 0; k < 8; k++) {
       const uint32_t rh = whi(v[k].re), ih = whi(v[k].im);
@@ -302,14 +318,10 @@ __device__ __forceinline__ bool pass(const PassParams<double>& p, void* smem, in
   // Transform (inverse, or the forward one of a kinetic pass), factors, transform (forward, or
   // the inverse one of a kinetic pass): one copy of the transform's code for both, because
   // the instruction cache holds little more (two copies waited on instruction fetches).
-  int spoil = 0;  // a factor that is not finite spoils its tile
   const bool t0 = kin || (f & F_IFFT), t1 = kin || (f & F_FFT), mid = ph || kin || (t0 && t1);
 #pragma unroll 1
   for (int it = 0; it < 2; it++) {
-    if (it == 0 ? t0 : t1) {
-      ti.fft(x, tw, sc);
-      ex += sc.total - sc.first;
-    }
+    if (it == 0 ? t0 : t1) ti.fft(x, tw, shifts);
     if (it == 1 || !mid) continue;
     // the factors of the middle of the pass, and the new bound for the transform after it
     if (swap) exchange(x);
@@ -345,7 +357,7 @@ __device__ __forceinline__ bool pass(const PassParams<double>& p, void* smem, in
 #pragma unroll
       for (int k = 0; k < 8; k++) x[k] = ti.at(ti.t + k * TL);
     }
-    uint32_t any = 0;
+    any = bad ? 0x80000000u : 0u;  // a factor that is not finite spoils its line
     L = 0;
 #pragma unroll
     for (int k = 0; k < 8; k++) {
@@ -353,38 +365,41 @@ __device__ __forceinline__ bool pass(const PassParams<double>& p, void* smem, in
       any |= ar | ai;
       L += fx_mag_int<kFxPassSum>(ar) + fx_mag_int<kFxPassSum>(ai);
     }
+    ti.line_bounds(any, L, red[R3], red[0]);
+    if (any >> 31) kind = SPOIL;
     if (t0 && t1) {
       // the transform before has changed the bounds: a new scale
-      const uint32_t Lm = ti.sum(L, any, red[1], redm[2]);
-      sc = fx_schedule<LOGN>(65 - __clz((int)any), fx_sum_bits<kFxPassSum>(Lm));
-      ex += sc.first;
+      const FxSchedule sc = fx_schedule<LOGN>(65 - __clz((int)(any & 0x7fffffffu)), fx_sum_bits<kFxPassSum>(L));
+      ex += sc.total;
+      shifts = packed(sc);
 #pragma unroll
       for (int k = 0; k < 8; k++) x[k] = mk(shift_jam(x[k].re, sc.first), shift_jam(x[k].im, sc.first));
     }
-    if (ph || kin) spoil = __syncthreads_or(bad);
     swap = kin;
     if (swap) exchange(x);
   }
   if (swap) exchange(x);
   if (kin) ex -= p.g.ln[0] + p.g.ln[1] + p.g.ln[2];  // 1/N
-  if (!OBS && out_fx) {
-    // each thread's eight points shifted up together, so that the code bits cost nothing of
-    // their largest
-    uint32_t any = 0;
+  // what a line that is all zero, or not finite, is stored with
+  if (kind == ZERO) {
+    ex = -2 * kFxNan;
 #pragma unroll
-    for (int k = 0; k < 8; k++) any |= absh(x[k].re) | absh(x[k].im);
-    const uint32_t up = (uint32_t)max(__clz((int)any) - 1, 0);
-    int32_t code = ex - (int32_t)up + kFxBias;
-    if (code <= 0 || spoil) {
-      code = spoil ? kFxNan : 0;
-    }
+    for (int k = 0; k < 8; k++) x[k] = mk((int64_t)0, (int64_t)0);
+  }
+  if (kind == SPOIL) ex = 2 * kFxNan;
+  int64_t step;
+  cx<double>* dst = p.out + ti.base(p.log_inner, tile, step);
+  if (!OBS && out_fx) {
+    // each point shifted up as far as it goes, so that the code bits cost nothing of it
 #pragma unroll
     for (int k = 0; k < 8; k++) {
+      const uint32_t up = (uint32_t)__clz((int)(absh(x[k].re) | absh(x[k].im))) - 1u;  // |x| < 2^63
+      const int32_t code = min(max(ex + kFxBias - (int32_t)up, 0), kFxNan);
       const uint64_t re = (uint64_t)x[k].re << up, im = (uint64_t)x[k].im << up;
       const uint32_t rl = ((uint32_t)re & ~63u) | ((uint32_t)code >> 6), il = ((uint32_t)im & ~63u) | ((uint32_t)code & 63u);
       dst[k * step] = mk(__hiloint2double((int)(re >> 32), (int)rl), __hiloint2double((int)(im >> 32), (int)il));
     }
-    return true;
+    return;
   }
   const bool chk = ex < 200 || ex > 1900;  // the range of a double may be left
 #pragma unroll
@@ -394,11 +409,10 @@ __device__ __forceinline__ bool pass(const PassParams<double>& p, void* smem, in
     fx_to_double(x[k].im, ex, ih, il);
     cx<double> y = mk(__hiloint2double((int)rh, (int)rl), __hiloint2double((int)ih, (int)il));
     if (chk) y = scaled(x[k], ex - 1085);
-    if (spoil) y = mk(__longlong_as_double(0x7ff8000000000000ll), __longlong_as_double(0x7ff8000000000000ll));
+    if (kind == SPOIL) y = mk(__longlong_as_double(0x7ff8000000000000ll), __longlong_as_double(0x7ff8000000000000ll));
     if (!OBS || !(f & F_NO_STORE)) dst[k * step] = y;
     if (OBS) v[k] = y;
   }
-  return true;
 }
 
 // The tile's row of the observable sums (obs_line_row's line sums), from the thread's points
@@ -518,7 +532,7 @@ __global__ void __launch_bounds__(256, 3) k_pass_fx_obs(const PassParams<double>
   cx<double> v[8];
   load<LOGN, CONTIG>(p.in, p.log_inner, blockIdx.x, v);
   if ((p.flags & (F_IFFT | F_PHASE | F_FFT | F_KIN)) || !(p.flags & F_NO_STORE))
-    if (!pass<LOGN, CONTIG, true>(p, smem_raw, blockIdx.x, v)) return;
+    pass<LOGN, CONTIG, true>(p, smem_raw, blockIdx.x, v);
   obs_sums<LOGN, CONTIG>(p, smem_raw, blockIdx.x, v);
 }
 

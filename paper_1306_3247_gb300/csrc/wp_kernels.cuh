@@ -1242,7 +1242,7 @@ namespace fxp {
 template <int LOGN, bool CONTIG>
 __device__ __forceinline__ void load(const cx<double>* in, int log_inner, int64_t tile, cx<double> (&v)[8]);
 template <int LOGN, bool CONTIG, bool OBS>
-__device__ __forceinline__ bool pass(const PassParams<double>& p, void* smem, int64_t tile, cx<double> (&v)[8]);
+__device__ __forceinline__ void pass(const PassParams<double>& p, void* smem, int64_t tile, cx<double> (&v)[8]);
 }  // namespace fxp
 
 // E elements per thread; the block has at most 32 E threads, so a tile holds at most

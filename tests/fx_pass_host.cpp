@@ -7,6 +7,7 @@
 //   1 two passes: forward transform, the line stored in fixed point and loaded again,
 //     inverse transform (n times the input)
 //   2 a resident line: forward transform
+//   3 the line's integers as loaded from doubles, stored in fixed point and read point by point
 #define __host__
 #define __device__
 #define __forceinline__ inline
@@ -93,16 +94,11 @@ struct Line {
     stages(0, LOGN);
     ex += sc.total - sc.first;
   }
-  // stored as the passes store it between them, loaded with its new bounds, transformed
-  void store_and_pass() {
-    std::vector<uint32_t> w(4 * N);  // re lo, re hi, im lo, im hi
+  // the points as the passes store them between them: re lo, re hi, im lo, im hi
+  std::vector<uint32_t> stored() const {
+    std::vector<uint32_t> w(4 * N);
     for (int i = 0; i < N; i++) {
-      uint32_t any = 0;
-      for (int k = 0; k < 8; k++) {
-        const C& v = x[i % (N / 8) + k * (N / 8)];
-        any |= absh(v.re) | absh(v.im);
-      }
-      const int up = std::max(fx_clz(any) - 1, 0);
+      const int up = std::max(fx_clz(absh(x[i].re) | absh(x[i].im)) - 1, 0);
       const uint32_t code = (uint32_t)(ex - up + kFxBias);
       const uint64_t re = (uint64_t)x[i].re << up, im = (uint64_t)x[i].im << up;
       w[4 * i] = ((uint32_t)re & ~63u) | (code >> 6);
@@ -110,6 +106,11 @@ struct Line {
       w[4 * i + 2] = ((uint32_t)im & ~63u) | (code & 63u);
       w[4 * i + 3] = (uint32_t)(im >> 32);
     }
+    return w;
+  }
+  // loaded again with its new bounds, transformed
+  void store_and_pass() {
+    const std::vector<uint32_t> w = stored();
     auto mag = [](uint32_t h) { return h ^ (uint32_t)((int32_t)h >> 31); };
     uint32_t m = 0, any = 0, L = 0;
     for (int i = 0; i < N; i++) m = std::max(m, fx_code(w[4 * i], w[4 * i + 2]));
@@ -157,6 +158,24 @@ struct Line {
       stages(kFxMidLog, LOGN);
     }
   }
+  // the integers of doubles at the line's exponent, stored and read back each by itself
+  void points(std::vector<double>& d) {
+    uint32_t m = 0, hi, lo;
+    for (double v : d) {
+      words(v, hi, lo);
+      m = std::max(m, hi & 0x7fffffffu);
+    }
+    ex = (int32_t)(m >> 20);
+    for (int i = 0; i < N; i++) x[i] = {load(d[2 * i], (uint32_t)ex), load(d[2 * i + 1], (uint32_t)ex)};
+    const std::vector<uint32_t> w = stored();
+    for (int i = 0; i < N; i++) {
+      const int32_t e = (int32_t)fx_code(w[4 * i], w[4 * i + 2]) - kFxBias;
+      for (int k = 0; k < 2; k++) {
+        const int64_t v = fx_align(w[4 * i + 2 * k], (int32_t)w[4 * i + 2 * k + 1], 0);
+        d[2 * i + k] = std::ldexp((double)v, e - 1085);
+      }
+    }
+  }
   void scale() {
     ex += sc.total;
     bS -= sc.total;
@@ -175,6 +194,10 @@ struct Line {
 template <int LOGN>
 static int go(int cmd, std::vector<double>& d) {
   Line<LOGN> l;
+  if (cmd == 3) {
+    l.points(d);
+    return 0;
+  }
   if (cmd == 2) {
     l.resident(d);
   } else {
@@ -188,7 +211,7 @@ static int go(int cmd, std::vector<double>& d) {
 int main() {
   int32_t hdr[2];
   if (fread(hdr, sizeof(hdr), 1, stdin) != 1) return 2;
-  if (hdr[0] < 0 || hdr[0] > 2 || hdr[1] < 5 || hdr[1] > 13) return 2;
+  if (hdr[0] < 0 || hdr[0] > 3 || hdr[1] < 5 || hdr[1] > 13) return 2;
   std::vector<double> d(2 << hdr[1]);
   if (fread(d.data(), 8, d.size(), stdin) != d.size()) return 2;
   switch (hdr[1]) {

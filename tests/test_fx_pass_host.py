@@ -62,3 +62,14 @@ def test_passes(fx, logn):
 def test_resident_lines(fx, logn):
     for name, x in lines(1 << logn, np.random.default_rng(logn)):
         assert rel(fx(2, x), np.fft.fft(x.astype(np.clongdouble))) < 2e-16, name
+
+
+@pytest.mark.parametrize("logn", range(5, 12))
+def test_stored_points(fx, logn):
+    """A stored point keeps 57 bits of its own size (half the range of the six code bits of a
+    number with its leading bit at 62), whatever its neighbours', above the 62 bits of the
+    line; 2^-53 for the doubles it is read back as."""
+    n, rng = 1 << logn, np.random.default_rng(logn)
+    x = (rng.standard_normal(n) + 1j * rng.standard_normal(n)) * 2.0 ** rng.uniform(-40, 0, n)
+    err = np.abs(fx(3, x).astype(np.clongdouble) - x)
+    assert np.all(err < 2.0 ** -52 * np.abs(x) + 2.0 ** -61 * np.max(np.abs(x)))
