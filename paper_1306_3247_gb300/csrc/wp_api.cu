@@ -822,7 +822,6 @@ Res1dParams<T> res1d_params(wp_handle* h) {
   p.vgrid = h->vgrid;
   p.fixed = h->res_fixed ? 1 : 0;
   p.max_radix_log = h->res_max_radix_log;
-  p.Wst = tb[0].Wst;
   p.Krec[0] = tb[0].Kfull_rec;
   p.Krec[1] = tb[0].Khalf_rec;
   p.Wln = tb[0].Wln;
@@ -1533,7 +1532,7 @@ wp_status batch_issue(wp_batch* b, int64_t m) {
     const auto* prm = (const Res1dParams<T>*)c.dparams;
     const int ni = (int)c.idx.size();
     s2 = launch_rc(nullptr,
-                   c.fixed ? launch_res1d_fixed_batch<T>(prm, ni, c.logn, m, c.smem, st1)
+                   c.fixed ? launch_res1d_fixed_batch<T>(prm, ni, c.logn, m, st1)
                            : launch_res1d_batch<T>(prm, ni, c.nthreads, c.ept, m, c.smem, st1),
                    "batched 1-D kernel");
     if (s2 != WP_OK) return s2;

@@ -336,7 +336,6 @@ struct Res1dParams {
   const double* vgrid;       // static grid potential (observables; the phase is in S), or NULL
   int32_t fixed;             // compile-time line length (wp_line.cuh), n = 2^8 .. 2^14
   int32_t max_radix_log;     // largest butterfly of the run-time-length kernel (2 or 3)
-  const void* Wst;           // per-stage twiddle records (fixed)
   const TwE<T>* Krec[2];     // kinetic factors dt, dt/2 as records (fixed)
   const void* Wln;           // stage twiddles (fixed): records of the form, FxRec for complex128
   // complex128 (fixed): kinetic factors without 1/n and static phases (dt, dt/2) in fixed point
@@ -504,10 +503,10 @@ template <class T> int launch_fixed_grid_obs(const PassParams<T>& p, unsigned nt
 template <class T> int fixed_grid_obs_smem_limit_set(size_t smem);
 template <class T> int res1d_smem_limit_set(size_t smem);
 // fixed-length resident-line kernels (their own translation units, wp_res1d_*.cu)
-template <class T> int launch_res1d_fixed(const Res1dParams<T>& p, size_t smem, void* stream);
+template <class T> int launch_res1d_fixed(const Res1dParams<T>& p, void* stream);
 template <class T> int launch_res1d_fixed_batch(const Res1dParams<T>* params, int ninst, int logn, int64_t nsteps,
-                                                size_t smem, void* stream);
-template <class T> int res1d_fixed_smem_limit_set(size_t smem);
+                                                void* stream);
+template <class T> int res1d_fixed_smem_limit_set();
 
 // Handle access for the run-time compiled potentials (wp_jit.cu).
 wp_status handle_set_error(wp_handle* h, wp_status st, const char* msg);

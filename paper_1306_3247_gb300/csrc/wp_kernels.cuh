@@ -376,14 +376,14 @@ __device__ __forceinline__ cx<float> tw_apply(cx<float> v, const TwE<float>& e) 
   return INV ? cmulc2(v, e.h, e.l) : cmul2(v, e.h, e.l);
 }
 
-template <class T, int LOGN, int LOGC, int LS, int LOGNS, bool INV, int EPT = 8>
+template <class T, int LOGN, int LOGC, int LS, int LOGNS, bool INV>
 __device__ __forceinline__ void stage_fixed(cx<T>* s, const TwE<T>* __restrict__ tw, int tid) {
   constexpr int LR = wp_stage_radix_log(LOGN, LOGNS);
   constexpr int R = 1 << LR;
   constexpr int C = 1 << LOGC;
   constexpr int NR = 1 << (LOGN - LR);
-  constexpr int NT = (C << LOGN) / EPT;  // threads: EPT elements each
-  constexpr int B = EPT / R;
+  constexpr int NT = (C << LOGN) / 8;  // threads: eight elements each
+  constexpr int B = 8 / R;
   constexpr int NS = 1 << LOGNS;
   cx<T> v[B][R];
 #pragma unroll
@@ -413,14 +413,14 @@ __device__ __forceinline__ void stage_fixed(cx<T>* s, const TwE<T>* __restrict__
 
 // The FP64 stages in fused multiply-add form (wp_fft_f64.h): the same loads, stores and
 // stage plan; the butterflies read their twiddle records from the direction's table.
-template <int LOGN, int LOGC, int LS, int LOGNS, bool INV, int EPT = 8>
+template <int LOGN, int LOGC, int LS, int LOGNS, bool INV>
 __device__ __forceinline__ void stage_fixed_f64(cx<double>* s, const unsigned char* __restrict__ tab, int tid) {
   constexpr int LR = wp_stage_radix_log(LOGN, LOGNS);
   constexpr int R = 1 << LR;
   constexpr int C = 1 << LOGC;
   constexpr int NR = 1 << (LOGN - LR);
-  constexpr int NT = (C << LOGN) / EPT;  // threads: EPT elements each
-  constexpr int B = EPT / R;
+  constexpr int NT = (C << LOGN) / 8;  // threads: eight elements each
+  constexpr int B = 8 / R;
   constexpr int NS = 1 << LOGNS;
   constexpr int OFF = (INV ? wp_fma_dir_bytes(LOGN) : 0) + wp_fma_stage_offset(LOGN, LOGNS);
   constexpr int RB = wp_fma_rec_bytes(LR);
@@ -459,18 +459,15 @@ __device__ __forceinline__ void stage_fixed_f64(cx<double>* s, const unsigned ch
 }
 
 // tw: the per-stage records of the axis, 2^LOGN 16-byte entries; for FP64 the fused
-// multiply-add records of both directions follow them. FMA: use those (FP64 only; the
-// resident 1-D lines keep the product form, whose register needs fit their blocks).
-template <class T, int LOGN, int LOGC, int LS, bool INV, int LOGNS, int EPT = 8,
-          bool FMA = std::is_same<T, double>::value>
+// multiply-add records of both directions follow them, which its stages use.
+template <class T, int LOGN, int LOGC, int LS, bool INV, int LOGNS>
 __device__ __forceinline__ void fft_fixed(cx<T>* s, const TwE<T>* __restrict__ tw, int tid) {
   if constexpr (LOGNS < LOGN) {
-    if constexpr (FMA)
-      stage_fixed_f64<LOGN, LOGC, LS, LOGNS, INV, EPT>(s, reinterpret_cast<const unsigned char*>(tw + (1 << LOGN)),
-                                                       tid);
+    if constexpr (std::is_same<T, double>::value)
+      stage_fixed_f64<LOGN, LOGC, LS, LOGNS, INV>(s, reinterpret_cast<const unsigned char*>(tw + (1 << LOGN)), tid);
     else
-      stage_fixed<T, LOGN, LOGC, LS, LOGNS, INV, EPT>(s, tw + wp_stage_tw_offset(LOGN, LOGNS), tid);
-    fft_fixed<T, LOGN, LOGC, LS, INV, LOGNS + wp_stage_radix_log(LOGN, LOGNS), EPT, FMA>(s, tw, tid);
+      stage_fixed<T, LOGN, LOGC, LS, LOGNS, INV>(s, tw + wp_stage_tw_offset(LOGN, LOGNS), tid);
+    fft_fixed<T, LOGN, LOGC, LS, INV, LOGNS + wp_stage_radix_log(LOGN, LOGNS)>(s, tw, tid);
   }
 }
 

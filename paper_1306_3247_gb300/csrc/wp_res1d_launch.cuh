@@ -56,7 +56,7 @@ cudaError_t go(K kern, unsigned nlines, cudaStream_t st, A... args) {
 }
 
 template <class T, int LOGN>
-cudaError_t launch_n(const Res1dParams<T>& p, size_t, cudaStream_t st) {
+cudaError_t launch_n(const Res1dParams<T>& p, cudaStream_t st) {
   if constexpr (supported<T, LOGN>()) {
     constexpr int LOGR = cluster_log<LOGN>();
     using SH = line::Shape<T, LOGN, LOGR>;
@@ -66,7 +66,7 @@ cudaError_t launch_n(const Res1dParams<T>& p, size_t, cudaStream_t st) {
 }
 
 template <class T, int LOGN>
-cudaError_t launch_batch_n(const Res1dParams<T>* params, int ninst, int64_t nsteps, size_t, cudaStream_t st) {
+cudaError_t launch_batch_n(const Res1dParams<T>* params, int ninst, int64_t nsteps, cudaStream_t st) {
   if constexpr (supported<T, LOGN>()) {
     constexpr int LOGR = batch_cluster_log<LOGN>();
     using SH = line::Shape<T, LOGN, LOGR, true>;
@@ -76,7 +76,7 @@ cudaError_t launch_batch_n(const Res1dParams<T>* params, int ninst, int64_t nste
 }
 
 template <class T, int LOGN>
-cudaError_t set_limit(int) {
+cudaError_t set_limit() {
   if constexpr (supported<T, LOGN>()) {
     constexpr int LOGR = cluster_log<LOGN>(), LOGB = batch_cluster_log<LOGN>();
     const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
@@ -124,29 +124,29 @@ bool dispatch(int logn, F&& f) {
 #define WP_RES1D_TU(T)                                                                                 \
   namespace wp {                                                                                       \
   template <>                                                                                          \
-  int launch_res1d_fixed<T>(const Res1dParams<T>& p, size_t smem, void* stream) {                      \
+  int launch_res1d_fixed<T>(const Res1dParams<T>& p, void* stream) {                                   \
     cudaError_t e = cudaErrorInvalidConfiguration;                                                     \
     res1d_detail::dispatch(p.logn, [&](auto L) {                                                       \
-      e = res1d_detail::launch_n<T, decltype(L)::value>(p, smem, (cudaStream_t)stream);                \
+      e = res1d_detail::launch_n<T, decltype(L)::value>(p, (cudaStream_t)stream);                      \
     });                                                                                                \
     return e == cudaSuccess ? 0 : (int)e;                                                              \
   }                                                                                                    \
   template <>                                                                                          \
   int launch_res1d_fixed_batch<T>(const Res1dParams<T>* params, int ninst, int logn, int64_t nsteps,  \
-                                  size_t smem, void* stream) {                                         \
+                                  void* stream) {                                                      \
     if (ninst <= 0) return 0;                                                                          \
     cudaError_t e = cudaErrorInvalidConfiguration;                                                     \
     res1d_detail::dispatch(logn, [&](auto L) {                                                         \
-      e = res1d_detail::launch_batch_n<T, decltype(L)::value>(params, ninst, nsteps, smem,             \
+      e = res1d_detail::launch_batch_n<T, decltype(L)::value>(params, ninst, nsteps,                   \
                                                               (cudaStream_t)stream);                   \
     });                                                                                                \
     return e == cudaSuccess ? 0 : (int)e;                                                              \
   }                                                                                                    \
   template <>                                                                                          \
-  int res1d_fixed_smem_limit_set<T>(size_t smem) {                                                     \
+  int res1d_fixed_smem_limit_set<T>() {                                                                \
     cudaError_t e = cudaSuccess;                                                                       \
     for (int l = kRes1dLogMin; l <= kRes1dLogMax && e == cudaSuccess; l++)                             \
-      res1d_detail::dispatch(l, [&](auto L) { e = res1d_detail::set_limit<T, decltype(L)::value>((int)smem); }); \
+      res1d_detail::dispatch(l, [&](auto L) { e = res1d_detail::set_limit<T, decltype(L)::value>(); }); \
     return e == cudaSuccess ? 0 : (int)e;                                                              \
   }                                                                                                    \
   }
