@@ -1053,14 +1053,15 @@ wp_status fft_seq(wp_handle* h, int sign) {
 // first call that comes here, whatever ran in between, and cleared with that; a norm that is
 // not finite only by the run or observation that found it (norm = true).
 wp_status check_device_error(wp_handle* h, bool norm = true) {
-  int32_t err = 0;
-  int32_t* const dev = (int32_t*)((char*)h->ctrl + offsetof(Ctrl, err));
-  WP_CUDA(h, cudaMemcpyAsync(&err, dev, sizeof(err), cudaMemcpyDeviceToHost, h->stream));
+  Ctrl c{};
+  WP_CUDA(h, cudaMemcpyAsync(&c, h->ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, h->stream));
   WP_CUDA(h, cudaStreamSynchronize(h->stream));
-  if (err == 0 || (err == WP_ENONFINITE && !norm)) return WP_OK;
-  if (err == WP_ENONFINITE) return fail(h, WP_ENONFINITE, "norm is not finite");
-  WP_CUDA(h, cudaMemsetAsync(dev, 0, sizeof(err), h->stream));
-  return fail(h, (wp_status)err, "a device wait ran out: the state is not valid");
+  if (c.lost) {
+    WP_CUDA(h, cudaMemsetAsync((char*)h->ctrl + offsetof(Ctrl, lost), 0, sizeof(c.lost), h->stream));
+    return fail(h, WP_ETIMEOUT, "a device wait ran out: the state is not valid");
+  }
+  if (c.err == WP_ENONFINITE && norm) return fail(h, WP_ENONFINITE, "norm is not finite");
+  return WP_OK;
 }
 
 template <class T>
@@ -1610,10 +1611,11 @@ namespace wp {
 
 wp_status handle_set_error(wp_handle* h, wp_status st, const char* msg) { return fail(h, st, msg); }
 
-// What a kernel's raise_error does, from the host: for tests of the reporting, which cannot let
-// a device wait run out.
-wp_status handle_raise(wp_handle* h, int err) {
-  WP_CUDA(h, cudaMemcpyAsync((char*)h->ctrl + offsetof(Ctrl, err), &err, sizeof(int32_t), cudaMemcpyHostToDevice, h->stream));
+// What a kernel does when a bounded wait runs out, from the host: for tests of the reporting,
+// which cannot let a device wait run out.
+wp_status handle_lose_wait(wp_handle* h) {
+  const int32_t one = 1;
+  WP_CUDA(h, cudaMemcpyAsync((char*)h->ctrl + offsetof(Ctrl, lost), &one, sizeof(one), cudaMemcpyHostToDevice, h->stream));
   WP_CUDA(h, cudaStreamSynchronize(h->stream));
   return WP_OK;
 }

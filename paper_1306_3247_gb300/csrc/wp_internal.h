@@ -152,8 +152,9 @@ struct Ctrl {
   double t_tab;                  // time of the current potential tables
   double gphase[WP_MAX_GAUSS];   // f_g(t) tau / hbar for the Gaussian terms
   double gcoef[WP_MAX_GAUSS];    // f_g(t)
-  int32_t err;                   // worst error raised by a kernel (0 = none); WP_ETIMEOUT stays until read
+  int32_t err;                   // WP_ENONFINITE when a record's norm was not finite, cleared with the step index
   uint32_t prep_done;            // blocks of the current k_prep launch that have finished
+  int32_t lost;                  // a bounded wait ran out (the state is not valid); cleared by the host that reports it
 };
 
 // Potential descriptor as the kernels read it (same field meaning as wp_potential).

@@ -516,11 +516,6 @@ __device__ __forceinline__ void finish_obs(const double* qp, const double* qm, c
   if (lane < 16) rec[lane] = v;
 }
 
-// A kernel's error into the control block. A wait that ran out outranks a norm that is not
-// finite: the status codes are in this order.
-static_assert((int)WP_ETIMEOUT > (int)WP_ENONFINITE, "");
-__device__ __forceinline__ void raise_error(Ctrl* ctrl, wp_status st) { atomicMax(&ctrl->err, (int32_t)st); }
-
 // The record into the next slot of the run (the 32 lanes of one warp).
 __device__ __forceinline__ void publish_obs(const double* qp, const double* qm, const Geom& g, int autocorr, double t,
                                             int64_t step, int lane, Ctrl* ctrl, double* obs_out, int64_t cap) {
@@ -529,7 +524,7 @@ __device__ __forceinline__ void publish_obs(const double* qp, const double* qm, 
   if (slot < cap) {
     double* rec = obs_out + slot * 16;
     finish_obs(qp, qm, g, autocorr, t, step, lane, rec);
-    if (lane == 1 && !isfinite(rec[1])) raise_error(ctrl, WP_ENONFINITE);
+    if (lane == 1 && !isfinite(rec[1])) ctrl->err = WP_ENONFINITE;
   }
   if (lane == 0) ctrl->nobs = slot + 1;
 }
@@ -1904,9 +1899,7 @@ __global__ void k_set_step(Ctrl* c, int64_t step) {
   pass_begin();
   c->step = step;
   c->nobs = 0;
-  // a norm that was not finite is the run's that found it; a wait that ran out has spoilt the
-  // state and stays until the host has reported it
-  if (c->err == WP_ENONFINITE) c->err = 0;
+  c->err = 0;  // not `lost`: that stays until the host has reported it
 }
 
 __global__ void k_add_step(Ctrl* c, int64_t add) { c->step += add; }

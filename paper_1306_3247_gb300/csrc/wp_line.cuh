@@ -167,7 +167,7 @@ struct Line {
     for (int k = 0; k < (1 << 20); k++)
       if (try_wait(pair + (n & 1u), (n >> 1) & 1u)) return;
     lost = true;
-    raise_error(ctrl, WP_ETIMEOUT);
+    ctrl->lost = 1;
   }
 
   // (union, sum) of the line's (any, L), in every thread.

@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(256, Shape<float>::kMinBlocks)
       }
     s_ok = ok;
     if (!ok) {
-      raise_error(const_cast<Ctrl*>(p.ctrl), WP_ETIMEOUT);
+      const_cast<Ctrl*>(p.ctrl)->lost = 1;
       // let a late copy land before the block's shared memory is given up (bounded too)
       for (int it = 0; it < (1 << 22) && !mbar_try_wait(bar_s, 0); it++) {
       }

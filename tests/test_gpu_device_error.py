@@ -13,10 +13,10 @@ pytestmark = pytest.mark.gpu
 SHAPES = [(64,), (1024,), (4096,), (64, 128), (32, 32, 32)]
 
 
-def raise_error(h, status=WPK.WP_ETIMEOUT):
-    f = WPK.load_library()._ZN2wp12handle_raiseEP9wp_handlei
-    f.argtypes, f.restype = [ctypes.c_void_p, ctypes.c_int], ctypes.c_int
-    assert f(h, status) == WPK.WP_OK
+def raise_error(h):
+    f = WPK.load_library()._ZN2wp16handle_lose_waitEP9wp_handle
+    f.argtypes, f.restype = [ctypes.c_void_p], ctypes.c_int
+    assert f(h) == WPK.WP_OK
 
 
 def problem(n):
