@@ -366,6 +366,11 @@ __device__ __forceinline__ void tables(const Res1dParams<T>& p, double t, double
   }
 }
 
+// Thread q's part of the coefficients at time t (one copy of the sine's code beside the tables').
+static __device__ __noinline__ void record_coefs(const DevPot& pot, double t, double* fco, int q) {
+  if (q < pot.nterms) fco[q] = term_coef(pot.term[q], t);
+}
+
 // FP64 sums of the line in a fixed order into `out` (shared memory of block 0): the block's
 // warps in order, then (part: [R][NQ] in block 0, n: which of its two record mbarriers) the
 // blocks. used: the quantities to sum (a shuffle tree is five dependent FP64 adds, 320 clocks,
@@ -457,12 +462,23 @@ __device__ __forceinline__ void body(const Res1dParams<T>& p, unsigned char* sme
     cluster_sync();  // every block is there, its mbarriers ready
   }
   __syncthreads();  // the step index is read
+  const bool obs = !BATCH && p.obs;
+  // The coefficients at the time of a record, in fco[m & 1]: those of the last potential phase,
+  // or (a record of the state as it is, and after a kinetic half step) formed by the table warps
+  // while the others load or finish.
+  [[maybe_unused]] auto record_time = [&] { return p.g.t0 + (double)(s0 + m) * dt; };
+  [[maybe_unused]] const bool coefs = obs && !(vkv && m > 0);
+  static_assert(BATCH || SH::TW > 0, "");
   // One barrier of the block per phase: the tables of phase k are complete, and those of phase
   // k - 1 no longer read.
   if constexpr (SH::TW > 0) {
     if (t >= NT) {
       for (int64_t k = 0; k < nphase; k++) {
         make(k, t - NT, SH::TW, [] { asm volatile("bar.sync 2, %0;" ::"n"(SH::TW) : "memory"); });
+        __syncthreads();
+      }
+      if (coefs) {
+        record_coefs(*p.pot, record_time(), fco[m & 1], t - NT);
         __syncthreads();
       }
       __syncthreads();
@@ -635,27 +651,24 @@ __device__ __forceinline__ void body(const Res1dParams<T>& p, unsigned char* sme
       return v;
     }
   };
-  const bool obs = !BATCH && p.obs;
+  // The linear and constant terms of a record, alpha + beta i at grid point i: from the sums of
+  // x |psi|^2 and |psi|^2 they would cancel on a box far from the origin. The general terms
+  // follow below.
   [[maybe_unused]] const DevPot& pot = *p.pot;
-  [[maybe_unused]] const double tm0 = p.g.t0 + (double)(s0 + m) * dt;
-  // The potential of a record, point by point: its linear terms from the sums of x |psi|^2 and
-  // |psi|^2 would cancel on a box far from the origin. The general terms follow below.
-  [[maybe_unused]] double W[P];
+  [[maybe_unused]] const double tm0 = record_time();
+  [[maybe_unused]] const double* fr = fco[m & 1];
+  [[maybe_unused]] double alpha = 0.0, beta = 0.0;
+  if (coefs) __syncthreads();
   if (obs) {
-    ln.bar();
-    if (t < pot.nterms) fco[0][t] = term_coef(pot.term[t], tm0);
-    ln.bar();
-#pragma unroll
-    for (int k = 0; k < P; k++) W[k] = p.Vs[ln.point(k)];
     for (int e = 0; e < pot.nterms; e++) {
       if (!((p.plane_mask >> e) & 1u)) continue;
       const wp_pot_term& tm = pot.term[e];
-      const bool lin = tm.shape == WP_SHAPE_LINEAR;
-      const double f = lin ? fco[0][e] * tm.a[0] : fco[0][e], ctr = tm.c0[0] + tm.v[0] * tm0;
-#pragma unroll
-      for (int k = 0; k < P; k++) {
-        const double xi = p.g.xmin[0] + (double)ln.point(k) * p.g.dx[0];
-        W[k] = lin ? fma(f, xi - ctr, W[k]) : W[k] + f;
+      if (tm.shape == WP_SHAPE_LINEAR) {
+        const double fa = fr[e] * tm.a[0];
+        beta = fma(fa, p.g.dx[0], beta);
+        alpha = fma(fa, p.g.xmin[0] - (tm.c0[0] + tm.v[0] * tm0), alpha);
+      } else {
+        alpha += fr[e];
       }
     }
   }
@@ -674,7 +687,7 @@ __device__ __forceinline__ void body(const Res1dParams<T>& p, unsigned char* sme
       acc[Q_RHO] += rho;
       acc[Q_X] += xr;
       acc[Q_XX] += xi * xr;
-      acc[Q_V] += W[k] * rho;
+      acc[Q_V] += (p.Vs[i] + fma(beta, (double)i, alpha)) * rho;
       if (p.autocorr) {
         const cx<T> z = p.psi0[i];
         const double zr = to_f64(z.re), zi = to_f64(z.im);
@@ -694,7 +707,7 @@ __device__ __forceinline__ void body(const Res1dParams<T>& p, unsigned char* sme
         for (int e = 0; e < pot.nterms; e++) {
           if (!((p.gen_mask >> e) & 1u)) continue;
           const wp_pot_term& tm = pot.term[e];
-          W += fco[0][e] * ((tm.shape == WP_SHAPE_GAUSS) ? gauss_axis_factor(tm, 0, xi, tm0) : term_axis_part(tm, 0, xi, tm0));
+          W += fr[e] * ((tm.shape == WP_SHAPE_GAUSS) ? gauss_axis_factor(tm, 0, xi, tm0) : term_axis_part(tm, 0, xi, tm0));
         }
         acc[Q_V] += W * fma(re, re, im * im);
         const V first = x[0];
