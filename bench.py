@@ -45,15 +45,19 @@ from paper_1306_3247_gb300 import workloads as W  # noqa: E402
 
 METRIC = "grid-point·steps/s (256³ c128 plain vs batched c64) + served p50/p99 ms"
 UNIT = "grid-point·steps/s"
-# DRAM bytes (read + write) per launch of each pass class on the 256^3 workload, from one
-# ncu capture (dram__bytes_read.sum + dram__bytes_write.sum; of the FP64 passes for c128, which
-# swept the same state once a pass as the fixed-point ones do). Valid
+# DRAM bytes (read + write) per launch of each pass class on a 256^3 state, from one
+# ncu capture (dram__bytes_read.sum + dram__bytes_write.sum) of the kernels in use. Valid
 # for grid 256 only; any other grid reports null.
 TRAFFIC_256 = {
-    "c128": {"pass_contig": 480336128, "pass_strided": 472172288, "pass_kinetic": 477476096},
+    "c128": {"pass_contig": 483636224, "pass_strided": 477612576, "pass_kinetic": 479800320},
     "c64": {"pass_contig": 206836992, "pass_strided": 205500416, "pass_kinetic": 209300736},
     "c128f": {"pass_contig": 474867456, "pass_strided": 471806464, "pass_kinetic": 477838592},
 }
+
+
+# What bounds the dominant pass of each form (profiles/): achieved and peak are HBM rates for
+# all of them.
+BOUND = {"c128": "integer pipe and issue", "c128f": "fp32 pipe", "c64": "hbm"}
 
 
 def traffic_of(grid, precision, kernel_class):
@@ -443,7 +447,7 @@ def main():
     avg_s = dom_v["avg_ms"] / 1e3
     elem = 8 if args.precision == "c64" else 16
     achieved = 2 * npts * elem / avg_s / 1e9
-    roof = {"bound": "hbm", "kernel": dom_name, "achieved": achieved, "peak": pk["hbm_gbs"], "unit": "GB/s",
+    roof = {"bound": BOUND[args.precision], "kernel": dom_name, "achieved": achieved, "peak": pk["hbm_gbs"], "unit": "GB/s",
             "frac": achieved / pk["hbm_gbs"], "traffic": traffic_of(args.grid, args.precision, dom_name),
             "peak_source": src,
             "avg_launch_ms": dom_v["avg_ms"], "launches": dom_v["launches"]}
@@ -462,7 +466,7 @@ def main():
                          keep_state=ref_state is not None)
             kd = max(r["kernels"].items(), key=lambda kv: kv[1]["launches"] * kv[1]["avg_ms"])
             el = 8 if form == "c64" else 16
-            r["roofline"] = {"bound": "hbm", "kernel": kd[0],
+            r["roofline"] = {"bound": BOUND[form], "kernel": kd[0],
                              "achieved": 2 * npts * el / (kd[1]["avg_ms"] / 1e3) / 1e9, "peak": pk["hbm_gbs"],
                              "unit": "GB/s", "traffic": traffic_of(args.grid, form, kd[0]), "peak_source": src}
             r["roofline"]["frac"] = r["roofline"]["achieved"] / pk["hbm_gbs"]

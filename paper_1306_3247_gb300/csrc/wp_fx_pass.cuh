@@ -4,11 +4,12 @@
 // threads, n = 32..2048, the lengths whose stages unroll); those that form observable sums
 // add them up in FP64 from the results; passes that apply a grid potential stay in FP64.
 //
-// Bound by the integer pipe (64 lanes per clock; ncu on 256^3: 63-69 % busy, FP64 before
-// 92 %) and by instruction issue. Measured on the 256^3 barrier, CUDA events in the step, FP64
-// before, fixed point with the whole tile in shared memory, and these: FFT-only pass 617, 162,
-// 159 us; kinetic pass 1411, 333, 322; potential pass 1118, 352, 290. The FP64 pipe bounds the
-// sums of a record (86 % busy in the position sums, 489 us).
+// Bound by the integer pipe (64 lanes per clock; ncu on 256^3: 66-74 % busy, FP64 before
+// 92 %) and by instruction issue (65-68 %). Measured on the 256^3 barrier, CUDA events in the
+// step, FP64 before, fixed point with the whole tile in shared memory, in registers with one
+// exponent per tile, and these: FFT-only pass 617, 162, 159, 164 us; kinetic pass 1411, 333, 322,
+// 332; potential pass 1118, 352, 290, 265 (its lines lie within a warp: no block barrier). The FP64 pipe bounds the
+// sums of a record (86 % busy in the position sums, 488 us).
 //
 // In memory a state is complex128 at the ends of a chunk of steps and in fixed point between
 // its passes (F_IN_FX, F_OUT_FX): the conversions between doubles and integers are about
@@ -511,8 +512,8 @@ __device__ __forceinline__ void load(const cx<double>* in, int log_inner, int64_
   for (int k = 0; k < 8; k++) v[k] = q[k * step];
 }
 
-// Three blocks per SM (80 registers); with four (64, and x spilled) the step at 256^3 takes
-// 994 us against 960, at 1024 x 1024 80 against 74.
+// Three blocks per SM (80 registers); with four (64, and x spilled) the step at 256^3 took
+// 994 us against 960, at 1024 x 1024 80 against 74 (with one exponent per tile).
 template <int LOGN, bool CONTIG>
 __global__ void __launch_bounds__(256, 3) k_pass_fx(const PassParams<double> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];

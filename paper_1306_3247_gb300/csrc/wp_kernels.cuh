@@ -32,7 +32,7 @@ namespace wp {
 // kernel has completed and its writes are visible. Every thread of every such kernel waits,
 // so the order of the chain is kept; kernels launched plainly wait for everything before them.
 // Measured, plain launches -> these: complex64 64^3, 50 steps 406 -> 378 us, 1024 x 1024, 100
-// steps 3214 -> 3058; float-float 512 x 128, 40 steps 1749 -> 1635; complex128 1024 x 1024,
+// steps 3214 -> 3058; float-float 512 x 128, 40 steps 1708 -> 1584; complex128 1024 x 1024,
 // 50 steps 4035 -> 3917. Letting the next kernel come forward at once (a trigger here) puts
 // waiting blocks in the way of the tables on the side stream: 1834 against 1625 us for the
 // float-float case.
@@ -719,10 +719,13 @@ __device__ __forceinline__ cx<ff> apply_factor_rec(cx<ff> v, const TwE<ff>& a, c
 // complex64: v (a L) with one rounding per component, a and L on their grids (make_axis_rec,
 // make_line_rec): the products of high parts are multiples of 2^-23 and exact, the cross
 // terms, below 2^-11, carry the rest to 2^-35. 20 instructions; forming a L from full-length
-// parts by error-free products (apply_factor) takes 44, a fifth of the kinetic pass's. Measured:
-// 40 steps of the 256^3 barrier with records 10.54 -> 10.15 ms, 20 steps of 512 batched
-// instances 1.66 -> 1.55 ms; the error against FP64 after 300 to 1000 steps no larger (128^2
-// trap 5.6e-6 -> 5.3e-6, its norm 1.5e-6 -> -8e-8).
+// parts by error-free products (apply_factor, 2^-46) takes 44, a fifth of the kinetic pass's.
+// Measured: 40 steps of the 256^3 barrier with records 10.16 -> 9.80 ms, 20 steps of 512 batched
+// instances 1.64 -> 1.51 ms. Results are no less exact: against the complex128 form over nine
+// grids (64^2 to 256^3; trap, laser, moving, barrier), both orders and 100 to 50000 steps the
+// error is 0.75 to 1.04 times (0.94 in the mean) that with the full product (256^2 laser, 10000 steps 2.2e-5 ->
+// 1.8e-5; 64^2 trap, 50000 steps 4.3e-5 -> 3.5e-5) and the largest norm drift 1.7e-5 -> 2.4e-6:
+// 2^-35 is far below the rounding of v itself, whose bias the exact high products reduce.
 __device__ __forceinline__ cx<float> apply_factor_rec(cx<float> v, const TwE<float>& a, const TwE<float>& L) {
   const cx<float> Lf = mk(L.h.re + L.l.re, L.h.im + L.l.im);
   const cx<float> fh = mk(fmaf(a.h.re, L.h.re, -(a.h.im * L.h.im)), fmaf(a.h.re, L.h.im, a.h.im * L.h.re));

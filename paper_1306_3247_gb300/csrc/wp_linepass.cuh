@@ -11,9 +11,10 @@
 // 32-byte sector of each row; the 2048-point tiles of wp_kernels.cuh read half sectors at
 // 1024 complex64 points.
 //
-// Bound: issue slots of the FP32 pipe at states that stay in L2, memory beyond.
-// Measured a step against those tiles: complex64 1024 x 1024 44.8 -> 31.3 us (kinetic pass 24
-// -> 19.3, potential pass 18 -> 14.5), 512 x 512 23.4 -> 12.3, 512^3 3951 -> 3146; float-float
+// Bound at states that stay in L2: load latency and the shared-memory path, with 37 to 40 % of
+// the warps (ncu, complex64 1024 x 1024: kinetic pass 17.0 us, potential pass 14.3; issue 36 and
+// 40 %, 6 and 4 warps per issue on global loads); beyond, memory and, float-float, arithmetic.
+// Measured a step against those tiles: complex64 1024 x 1024 44.8 -> 31.3 us, 512 x 512 23.4 -> 12.3, 512^3 3951 -> 3146; float-float
 // 512 x 512 40.2 -> 29.0, 1024 x 1024 79.6 -> 68.4, 512^3 8569 -> 8192. At 2048 points, whose
 // strided tile was one column: complex64 2048 x 1024 115 -> 51 us, float-float 193 -> 129.
 #pragma once
