@@ -140,6 +140,14 @@ struct Tile {
       m = get<Max>(red);
     }
   }
+  static __device__ __forceinline__ void line_sum(uint32_t& L, uint32_t* red) {
+    L = warp_part<Add>(L);
+    if constexpr (!IN_WARP) {
+      put(L, red);
+      __syncthreads();
+      L = get<Add>(red);
+    }
+  }
   // (union, sum) of the line's (any, L)
   static __device__ __forceinline__ void line_bounds(uint32_t& any, uint32_t& L, uint32_t* ra, uint32_t* rl) {
     any = warp_part<Or>(any);
@@ -266,12 +274,12 @@ __device__ __forceinline__ void pass(const PassParams<double>& p, void* smem, in
 #pragma unroll
     for (int k = 0; k < 8; k++) {
       const uint32_t d = m - fx_code(wlo(v[k].re), wlo(v[k].im));
-      const uint32_t ar = fx_shr64(absh(whi(v[k].re)), 0u, d), ai = fx_shr64(absh(whi(v[k].im)), 0u, d);
-      any |= ar | ai;
-      L += fx_mag_int<kFxPassSum>(ar) + fx_mag_int<kFxPassSum>(ai);
+      L += fx_mag_int<kFxPassSum>(fx_shr64(absh(whi(v[k].re)), 0u, d)) +
+           fx_mag_int<kFxPassSum>(fx_shr64(absh(whi(v[k].im)), 0u, d));
     }
-    ti.line_bounds(any, L, red[R1], red[R2]);
-    const FxSchedule sc = fx_schedule<LOGN>(65 - __clz((int)any), fx_sum_bits<kFxPassSum>(L));
+    ti.line_sum(L, red[R1]);
+    // the largest points have their leading bit at 62
+    const FxSchedule sc = fx_schedule<LOGN>(64, fx_sum_bits<kFxPassSum>(L));
     ex = (int32_t)m - kFxBias + sc.total;  // that of the transform's results
     shifts = packed(sc);
     const uint32_t right = sc.first > 0 ? (uint32_t)sc.first : 0u, left = sc.first < 0 ? (uint32_t)-sc.first : 0u;

@@ -112,15 +112,13 @@ struct Line {
   void store_and_pass() {
     const std::vector<uint32_t> w = stored();
     auto mag = [](uint32_t h) { return h ^ (uint32_t)((int32_t)h >> 31); };
-    uint32_t m = 0, any = 0, L = 0;
+    uint32_t m = 0, L = 0;
     for (int i = 0; i < N; i++) m = std::max(m, fx_code(w[4 * i], w[4 * i + 2]));
     for (int i = 0; i < N; i++) {
       const uint32_t s = m - fx_code(w[4 * i], w[4 * i + 2]);
-      const uint32_t ar = fx_shr64(mag(w[4 * i + 1]), 0u, s), ai = fx_shr64(mag(w[4 * i + 3]), 0u, s);
-      any |= ar | ai;
-      L += fx_mag_int<kFxPassSum>(ar) + fx_mag_int<kFxPassSum>(ai);
+      L += fx_mag_int<kFxPassSum>(fx_shr64(mag(w[4 * i + 1]), 0u, s)) + fx_mag_int<kFxPassSum>(fx_shr64(mag(w[4 * i + 3]), 0u, s));
     }
-    sc = fx_schedule<LOGN>(65 - fx_clz(any), fx_sum_bits<kFxPassSum>(L));
+    sc = fx_schedule<LOGN>(64, fx_sum_bits<kFxPassSum>(L));
     ex = (int32_t)m - kFxBias + sc.first;
     const uint32_t right = sc.first > 0 ? (uint32_t)sc.first : 0u, left = sc.first < 0 ? (uint32_t)-sc.first : 0u;
     for (int i = 0; i < N; i++) {
