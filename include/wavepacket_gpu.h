@@ -55,10 +55,10 @@ typedef enum {
  *                 significant bits) on the FP32 pipes, which GB300 runs about 58x faster
  *                 than FP64; 16 bytes per point in HBM. States enter and leave as
  *                 complex128. Where WP_C128 runs in fixed point it is as fast or faster (us a
- *                 step on GB300, C128 / F32X2: 256^3 939 / 995, 64^3 27 / 37, 1-D 1024 points
+ *                 step on GB300, C128 / F32X2: 256^3 934 / 995, 64^3 27 / 37, 1-D 1024 points
  *                 7.3 / 9.9) and rounds less; F32X2 is the faster one with a grid potential
- *                 (256^3 2337 / 1130, 1024 x 1024 179 / 79), on 1024 x 1024 and 2048 x 1024
- *                 (70 / 63, 135 / 126) and on axes below 32 points (16^3 49 / 38). */
+ *                 (256^3 2339 / 1132, 1024 x 1024 179 / 79), on 1024 x 1024 and 2048 x 1024
+ *                 (70 / 63, 133 / 126) and on axes below 32 points (16^3 50 / 38). */
 typedef enum { WP_C128 = 0, WP_C64 = 1, WP_C128_F32X2 = 2 } wp_precision;
 
 /* Operator order of one step (eq. (splitop)).

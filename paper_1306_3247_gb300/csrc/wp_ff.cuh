@@ -1,8 +1,8 @@
 // Float-float ("FP32 pair") real type for the complex128-accuracy form on GB300.
 //
 // GB300 executes FP64 at about 1/58 of its FP32 rate (measured: 1.2 vs 70 TFLOP/s), so passes in
-// FP64 are bound by that pipe: 4.0 ms per 256^3 step, against 1.03 in this form. The complex128
-// form's 64-bit fixed point (wp_fx.h) takes 0.95 and rounds less. A value here is the unevaluated sum hi + lo
+// FP64 are bound by that pipe: 4.0 ms per 256^3 step, against 1.02 in this form. The complex128
+// form's 64-bit fixed point (wp_fx.h) takes 0.94 and rounds less. A value here is the unevaluated sum hi + lo
 // of two floats (|lo| <= ulp(hi)/2), about 48 significant bits. Sums use Knuth's
 // two-sum of the high parts plus the low parts and one renormalisation; products use
 // Dekker's exact product through an FMA (error-free transformations, Dekker 1971, Knuth

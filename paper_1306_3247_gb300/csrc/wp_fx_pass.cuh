@@ -4,11 +4,11 @@
 // threads, n = 32..2048, the lengths whose stages unroll); those that form observable sums
 // add them up in FP64 from the results; passes that apply a grid potential stay in FP64.
 //
-// Bound by the integer pipe (64 lanes per clock; ncu on 256^3: 66-74 % busy, FP64 before
+// Bound by the integer pipe (64 lanes per clock; ncu on 256^3: 66-72 % busy, FP64 before
 // 92 %) and by instruction issue (65-68 %). Measured on the 256^3 barrier, CUDA events in the
 // step, FP64 before, fixed point with the whole tile in shared memory, in registers with one
-// exponent per tile, and these: FFT-only pass 617, 162, 159, 164 us; kinetic pass 1411, 333, 322,
-// 332; potential pass 1118, 352, 290, 265 (its lines lie within a warp: no block barrier). The FP64 pipe bounds the
+// exponent per tile, and these: FFT-only pass 617, 162, 159, 162 us; kinetic pass 1411, 333, 322,
+// 330; potential pass 1118, 352, 290, 265 (its lines lie within a warp: no block barrier). The FP64 pipe bounds the
 // sums of a record (86 % busy in the position sums, 488 us).
 //
 // In memory a state is complex128 at the ends of a chunk of steps and in fixed point between
